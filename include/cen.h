@@ -351,7 +351,9 @@ int cen_job_copy_signs(const cen_job *job, uint32_t *words);
 #define CEN_PARAM_LEVEL_BUDGET 4 /* max bytes of one per-level bit array [n][wave words] (default 2^30) */
 #define CEN_PARAM_SAMPLER 5      /* 0: balanced bidirectional search, one CTA per sample, with the
                                     bit-parallel sampler for what exceeds its per-CTA limits (default);
-                                    1: bit-parallel waves only.  Hyper-edges are identical. */
+                                    1: bit-parallel waves only.  Hyper-edges are identical.  On graphs of
+                                    up to 2^24 nodes the searches keep their state in shared memory;
+                                    those that outgrow it use the global-memory workspace below. */
 #define CEN_PARAM_BIDIR_BUDGET 6 /* device bytes for the bidirectional sampler's per-CTA workspace,
                                     >= 2^20 (default 2^34); fewer CTAs run when it is small.  One CTA
                                     needs 8 h + 16 H + 28 q bytes, plus 32,800 with warp searches
@@ -360,20 +362,23 @@ int cen_job_copy_signs(const cen_job *job, uint32_t *words);
 #define CEN_PARAM_BIDIR_QUEUE 7  /* nodes one CTA may hold per ball or cone side, 16 .. 2^27 (default
                                     2^16, at most n); larger searches go to the bit-parallel sampler */
 #define CEN_PARAM_BIDIR_TABLE 8  /* entries of each CTA's small node table: a power of two in
-                                    2^10 .. 2^24 (at most H / 2), 0 for none (searches use the large
-                                    table of H entries only), or -1 (default) to size all CTAs' small
-                                    tables to about 80 MiB so that they stay in L2; a search that
-                                    fills half of it moves to the large table.  With -1, once a call
-                                    of 1,024 or more samples sees most searches move, later jobs on
-                                    the graph use no small table */
+                                    2^10 .. 2^24 (at most H / 2) or 0 for none (searches use the large
+                                    table of H entries only); either way every search uses the tables
+                                    in global memory.  -1 (default): searches start in shared memory
+                                    where they can, and the small tables of those that cannot are
+                                    sized to about 80 MiB in all so that they stay in L2; a search
+                                    that fills half of its small table moves to the large one.  With
+                                    -1, once a call of 1,024 or more samples sees most searches move,
+                                    later jobs on the graph use no small table */
 #define CEN_PARAM_BIDIR_WARPS 9  /* 1: each warp of a CTA searches samples alone with a 1,024-entry
                                     node table, and a second launch searches with whole CTAs those it
                                     hands on (a level of more than 2,048 arcs to expand, more than 512
                                     nodes, or more than 64 levels a side); 0: every sample is searched
-                                    by a whole CTA; -1 (default): 0 on graphs whose degrees have
-                                    E[d^2]/E[d] > 256 (frontiers that soon outgrow a warp), else 1
-                                    until a call of 1,024 or more samples hands more than 30% on,
-                                    then 0 for later jobs on the graph.  Queues of fewer than 1,024
+                                    by a whole CTA; -1 (default): 0 while the CTAs' searches start in
+                                    shared memory and on graphs whose degrees have E[d^2]/E[d] > 256
+                                    (frontiers that soon outgrow a warp), else 1 until a call of 1,024
+                                    or more samples hands more than 30% on, then 0 for later jobs on
+                                    the graph.  Queues of fewer than 1,024
                                     nodes use CTA searches only */
 int cen_job_set_param(cen_job *job, int32_t param, double value);
 /* Releases the device memory the library keeps for reuse once jobs end: idle
@@ -385,9 +390,10 @@ int cen_release_cached(void);
 /* How the job's samples were drawn so far: samples the bidirectional search
  * left whole to the bit-parallel sampler (*deferred_search), samples whose walk
  * it left to it (*deferred_walk), searches that outgrew the small node table
- * (*migrated), the CTAs (slots) the bidirectional search runs on (0 before
- * its first use), and the warp searches handed on to whole CTAs because a
- * level, the node count or the depth was too large for one warp (*escalated).
+ * or the shared memory of a wide CTA (*migrated), the CTAs (slots) the
+ * bidirectional search has global workspace for (0 before its first use), and
+ * the warp searches handed on to whole CTAs because a level, the node count or
+ * the depth was too large for one warp (*escalated).
  * Any pointer may be NULL. */
 int cen_job_sampler_info(const cen_job *job, uint64_t *deferred_search, uint64_t *deferred_walk, uint64_t *migrated,
                          int32_t *slots, uint64_t *escalated);

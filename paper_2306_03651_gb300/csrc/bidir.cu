@@ -17,6 +17,15 @@
 // node, so these counts equal a full BFS's wherever the walk reads them, and
 // which side grew when changes only the cost.
 //
+// Searches run at several sizes, each a persistent launch that takes up what
+// the one before it handed on.  By default they start in shared memory
+// (bidir_log.cuh): CTAs of 128, 512 and 1,024 threads whose node table, queues
+// and counts fit there, for graphs of up to 2^24 nodes.  What outgrows those
+// (deep searches such as a rewired grid's, or 2^32 paths) is searched with the
+// tables in global memory, as everything is on larger graphs or when a table
+// size is set.  A graph whose searches mostly outgrow a size skips it from the
+// next call on.  The rest of this comment describes the global-memory form.
+//
 // Two granularities run in two persistent launches of 128-thread CTAs.  In
 // the first, each warp takes sample ids from a counter and searches on its
 // own ("warp search"): no CTA barrier, a private node table of kWarpTable
@@ -41,7 +50,9 @@
 // count reaching 2^64 or a full member arena ("walk" deferral, distance
 // known).  A cone side is part of its ball, so it always fits.
 #include <algorithm>
+#include <cstddef>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "job.cuh"
@@ -57,6 +68,7 @@ constexpr int kWarpLevels = 64;     // levels per side of a warp search
 constexpr int kBiHeavy = 256;       // rows longer than this are scanned by the whole search group
 constexpr uint32_t kEpochMax = (1u << 16) - 1;
 constexpr int kWarpLevelArcs = 2048; // a warp search hands on a level with more arcs to expand
+constexpr uint64_t kWideMost = 1024;  // fewer left searches than this go to wide CTAs
 constexpr int kBiCtaPerSM = 16;      // resident CTAs per SM (32 registers)
 constexpr int kBiWarpCtaPerSM = 12;  // warp-search CTAs per SM (40 registers: fewer spills, measured faster)
 
@@ -507,6 +519,7 @@ __device__ __forceinline__ bool row_has(const int32_t *__restrict__ c, int64_t e
 
 struct BiArgs {
   int32_t n;
+  int64_t nnz;
   const int64_t *off, *roff;
   const int32_t *col, *rcol;
   SampleKey key;  // Philox key and the map from store positions to sample ids
@@ -525,9 +538,11 @@ struct BiArgs {
   uint64_t *tabw;     // [slots][4][kWarpTable] node tables of the warp searches (null: CTA searches only)
   uint32_t *epw;      // [slots][4][2]: their epochs
   int64_t WQ;         // entries of each list of a warp search
-  uint64_t *big;      // [count]: relative ids of the searches the warp kernel handed on
-  const uint64_t *list;                   // list mode: relative sample ids, one CTA search each
+  unsigned long long *next;               // the launch's work counter
+  const uint64_t *list;                   // list mode: relative sample ids, one search each
   const unsigned long long *list_count;   // list mode: their number (device)
+  uint64_t *out;                          // [count]: relative ids of the searches the launch hands on
+  unsigned long long *out_count;
   int32_t *ps, *pt, *pd;
   int *bmax;
   int32_t *arena;
@@ -1036,11 +1051,34 @@ __global__ void __launch_bounds__(kBiThreads, kBiCtaPerSM) k_bidir(BiArgs A) {
   if (tid == 0) s_arcs = 0;
   for (;;) {
     __syncthreads();
-    if (tid == 0) s_item = atomicAdd(LIST ? &A.ctl->bignext : &A.ctl->next, 1ull);
+    if (tid == 0) s_item = atomicAdd(A.next, 1ull);
     __syncthreads();
     const unsigned long long i = s_item;
     if (i >= count) break;
     bi_search<kBiThreads, kBiMaxLevels>(A, sh, cw, LIST ? A.list[i] : i);
+    if (tid == 0) s_arcs += sh.arcs;
+  }
+  if (tid == 0 && s_arcs) atomicAdd(A.units, s_arcs * 12ull);
+}
+
+// The listed searches by wide CTAs, for a list of few: so that the last, large
+// searches of a call do not run on at 128 threads each while the rest of the
+// chip is idle.
+constexpr int kWideThreads = 1024;
+__global__ void __launch_bounds__(kWideThreads, 1) k_bidir_wide(BiArgs A) {
+  __shared__ BiSh<kBiMaxLevels, kWideThreads / 32> sh;
+  __shared__ unsigned long long s_item, s_arcs;
+  const int tid = threadIdx.x;
+  const BiWork cw = cta_work(A);
+  const unsigned long long count = *(volatile const unsigned long long *)A.list_count;
+  if (tid == 0) s_arcs = 0;
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) s_item = atomicAdd(A.next, 1ull);
+    __syncthreads();
+    const unsigned long long i = s_item;
+    if (i >= count) break;
+    bi_search<kWideThreads, kBiMaxLevels>(A, sh, cw, A.list[i]);
     if (tid == 0) s_arcs += sh.arcs;
   }
   if (tid == 0 && s_arcs) atomicAdd(A.units, s_arcs * 12ull);
@@ -1078,13 +1116,13 @@ __global__ void __launch_bounds__(kBiThreads, kBiWarpCtaPerSM) k_bidir_warp(BiAr
   unsigned long long arcs = 0;
   for (;;) {
     unsigned long long jr = 0;
-    if (lane == 0) jr = atomicAdd(&A.ctl->next, 1ull);
+    if (lane == 0) jr = atomicAdd(A.next, 1ull);
     jr = __shfl_sync(0xffffffffu, jr, 0);
     if (jr >= A.count) break;
     const int r = bi_search<32, kWarpLevels>(A, sh[wid], ww, jr);
     if (lane == 0) {
       if (r == kSearchBig)
-        A.big[atomicAdd(&A.ctl->nbig, 1ull)] = jr;
+        A.out[atomicAdd(A.out_count, 1ull)] = jr;
       else
         arcs += sh[wid].arcs;
     }
@@ -1094,6 +1132,20 @@ __global__ void __launch_bounds__(kBiThreads, kBiWarpCtaPerSM) k_bidir_warp(BiAr
   __syncthreads();
   if (tid == 0 && s_arcs) atomicAdd(A.units, s_arcs * 12ull);
 }
+
+#include "bidir_log.cuh"
+
+// The three sizes of shared-memory search.  Measured (R-MAT 18, 65,536 pairs,
+// against 5.33 ms with the tables in global memory): small 1.38 ms for all but
+// 3% of the searches, wide 0.39 ms for all but one of those, huge 0.10 ms.  The
+// small one is bound by instruction issue and the latency of short phases: 10
+// CTAs of 128 threads per SM took 1.38 ms, 9 took 1.44 and 7 (with a table of
+// 2,048 entries) 1.68; 64-thread CTAs 1.57.  A level of more than 65,536 arcs
+// goes to a wide CTA: at 32,768 the small launch falls to 1.29 ms and the wide
+// one rises to 0.60.
+using LogSmall = LogCfg<128, 1536, 1100, 1344, 65536, 10>;
+using LogWide = LogCfg<512, 7168, 5600, 8192, (1 << 24) - 1, 2>;
+using LogHuge = LogCfg<1024, 15360, 12288, 18432, (1 << 24) - 1, 1>;
 
 // ------------------------------------------------------------------ host
 int bidir_resident_slots() { return resident_grid((const void *)k_bidir<false>, kBiThreads); }
@@ -1140,7 +1192,7 @@ void bidir_give(std::unique_ptr<BiWS> w) {
   if (!w) return;
   // the job's stream may be gone before these buffers are: free them in order on the legacy stream
   for (DevBuf *b : {&w->tab1, &w->tab2, &w->lists, &w->sig, &w->epochs, &w->ctl, &w->aoff, &w->dsearch, &w->dwalk,
-                    &w->arena, &w->tabw, &w->epw, &w->big})
+                    &w->arena, &w->tabw, &w->epw, &w->big, &w->far})
     b->st = nullptr;
   BiCache &c = bi_cache();
   std::lock_guard<std::mutex> lk(c.mu);
@@ -1160,6 +1212,7 @@ BiArgs bidir_args(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap) 
   BiWS &w = *job->bws;
   BiArgs a;
   a.n = g->n;
+  a.nnz = g->nnz;
   a.off = g->off.as<int64_t>();
   a.col = g->col.as<int32_t>();
   a.roff = g->in_off();
@@ -1178,9 +1231,11 @@ BiArgs bidir_args(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap) 
   a.tabw = w.WQ ? w.tabw.as<uint64_t>() : nullptr;
   a.epw = w.WQ ? w.epw.as<uint32_t>() : nullptr;
   a.WQ = w.WQ;
-  a.big = w.big.as<uint64_t>();
+  a.next = nullptr;
   a.list = nullptr;
   a.list_count = nullptr;
+  a.out = nullptr;
+  a.out_count = nullptr;
   a.ps = job->ps.as<int32_t>();
   a.pt = job->pt.as<int32_t>();
   a.pd = job->pd.as<int32_t>();
@@ -1196,23 +1251,94 @@ BiArgs bidir_args(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap) 
 }
 }  // namespace
 
-void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap) {
+// Launches k_bidir_log<C> over every sample, or (list) over the listed ones.
+template <class C>
+static void log_launch(cen_job *job, const BiArgs &a, uint64_t count) {
+  const size_t smem = sizeof(LogSh<C>);
+  const void *kernel = a.list ? (const void *)k_bidir_log<C, true> : (const void *)k_bidir_log<C, false>;
+  allow_shared(kernel, smem);
+  const int grid = (int)std::min<uint64_t>(count, (uint64_t)sm_count() * C::CTAS);
+  launch(&job->stats, K_BIDIR, job->st, [&] {
+    if (a.list)
+      k_bidir_log<C, true><<<grid, C::T, smem, job->st>>>(a);
+    else
+      k_bidir_log<C, false><<<grid, C::T, smem, job->st>>>(a);
+  });
+}
+
+bool bidir_shared_ok(int32_t n) { return n <= kLogMaxNodes; }
+
+// The launches of one call search in turn what the one before handed on: the
+// list's length is read on the device.  Stage k counts its items in
+// ctl->next[k] and what it hands on in ctl->nout[k]; the lists alternate
+// between two buffers.
+static void next_stage(cen_job *job, BiArgs &a, int stage) {
+  BiWS &w = *job->bws;
+  BiCtl *ctl = w.ctl.as<BiCtl>();
+  a.list = stage ? a.out : nullptr;
+  a.list_count = stage ? &ctl->nout[stage - 1] : nullptr;
+  a.next = &ctl->next[stage];
+  a.out = (stage & 1 ? w.far : w.big).as<uint64_t>();
+  a.out_count = &ctl->nout[stage];
+}
+
+// Searches every sample of the call; what is left after the launches made here
+// (none after a launch with the tables in global memory) is listed, its number
+// in ctl->nout[*stages - 1].
+void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages) {
   BiWS &w = *job->bws;
   cudaStream_t st = job->st;
   CEN_CK(cudaMemsetAsync(w.ctl.p, 0, sizeof(BiCtl), st));
   BiArgs a = bidir_args(job, j0, count, arena_cap);
   const int grid = (int)std::min<uint64_t>((uint64_t)w.nslots, count);
-  if (!w.WQ) {
-    launch(&job->stats, K_BIDIR, st, [&] { k_bidir<false><<<grid, kBiThreads, 0, st>>>(a); });
-    return;
+  int stage = 0;
+  if (w.WQ) {
+    next_stage(job, a, stage++);
+    const int wgrid = std::max(1, std::min(grid, resident_grid((const void *)k_bidir_warp, kBiThreads)));
+    launch(&job->stats, K_BIDIR, st, [&] { k_bidir_warp<<<wgrid, kBiThreads, 0, st>>>(a); });
   }
-  // warp searches, then CTA searches of what they handed on (the list's
-  // length is read on the device, so no host round trip separates the two)
-  const int wgrid = std::max(1, std::min(grid, resident_grid((const void *)k_bidir_warp, kBiThreads)));
-  launch(&job->stats, K_BIDIR, st, [&] { k_bidir_warp<<<wgrid, kBiThreads, 0, st>>>(a); });
-  a.list = w.big.as<uint64_t>();
-  a.list_count = &w.ctl.as<BiCtl>()->nbig;
-  launch(&job->stats, K_BIDIR, st, [&] { k_bidir<true><<<grid, kBiThreads, 0, st>>>(a); });
+  next_stage(job, a, stage++);
+  switch (w.tier) {
+    case kTierSmall:
+      log_launch<LogSmall>(job, a, count);
+      next_stage(job, a, stage++);
+      [[fallthrough]];
+    case kTierWide:
+      log_launch<LogWide>(job, a, count);
+      break;
+    default:
+      launch(&job->stats, K_BIDIR, st, [&] {
+        if (a.list)
+          k_bidir<true><<<grid, kBiThreads, 0, st>>>(a);
+        else
+          k_bidir<false><<<grid, kBiThreads, 0, st>>>(a);
+      });
+  }
+  *stages = stage;
+}
+
+// The `left` searches that bidir_launch's stages handed on.  A few (the last,
+// large ones of a call) go to CTAs of 1,024 threads, with their state in shared
+// memory if it fits and in global memory if not, so that they do not run on at
+// 128 threads each while the rest of the chip is idle; many go to the 128-thread
+// CTAs with the tables in global memory.
+void bidir_launch_rest(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages, uint64_t left) {
+  BiWS &w = *job->bws;
+  cudaStream_t st = job->st;
+  BiArgs a = bidir_args(job, j0, count, arena_cap);
+  int stage = *stages;
+  next_stage(job, a, stage - 1);
+  next_stage(job, a, stage++);
+  if (left < kWideMost) {
+    log_launch<LogHuge>(job, a, left);
+    next_stage(job, a, stage++);
+    const int grid = (int)std::min<uint64_t>(std::min<uint64_t>((uint64_t)w.nslots, left), (uint64_t)sm_count());
+    launch(&job->stats, K_BIDIR, st, [&] { k_bidir_wide<<<grid, kWideThreads, 0, st>>>(a); });
+  } else {
+    const int grid = (int)std::min<uint64_t>((uint64_t)w.nslots, left);
+    launch(&job->stats, K_BIDIR, st, [&] { k_bidir<true><<<grid, kBiThreads, 0, st>>>(a); });
+  }
+  *stages = stage;
 }
 
 }  // namespace cen

@@ -259,6 +259,9 @@ inline void launch(Stats *S, int cls, cudaStream_t st, F &&f) {
 // Blocks of `block` threads that are resident at once on the current device
 // (SM count x blocks per SM for this kernel), cached per kernel.
 int resident_grid(const void *kernel, int block);
+// Lets `kernel` take `bytes` of dynamic shared memory on the current device
+// (once per device and kernel).
+void allow_shared(const void *kernel, size_t bytes);
 // Page-locked host buffers, reused across jobs (capacity in *cap, >= bytes).
 // A buffer is given back only once no copy into or out of it is in flight.
 void *pinned_take(size_t bytes, size_t *cap);
@@ -325,6 +328,9 @@ struct cen_graph {
   // Set once most bidirectional searches on this graph outgrew their node
   // table: later jobs (without an explicit table size) use the large table only.
   mutable std::atomic<bool> bidir_table_off{false};
+  // Where CTA searches on this graph start (kTier*): raised once a call handed
+  // most of its searches on.
+  mutable std::atomic<int> bidir_tier{0};
   // Set once a call handed more than 30% of its warp searches on to CTAs:
   // later jobs (without an explicit setting) search with whole CTAs only.
   mutable std::atomic<bool> bidir_warps_off{false};

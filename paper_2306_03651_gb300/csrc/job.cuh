@@ -55,20 +55,25 @@ struct WaveWS {
 // cone lists, heavy rows, crossing-arc tails and heads) and H2 path counts.
 // Nothing in it grows with the graph.
 struct BiCtl {
-  unsigned long long next;     // next sample, relative to the launch's first
+  unsigned long long next[5];  // next sample (or list entry) of each launch of a call
+  unsigned long long nout[5];  // searches each launch handed on to the next
   unsigned long long cursor;   // arena entries reserved
   unsigned long long nsearch;  // samples left whole to the bit-parallel sampler
   unsigned long long nwalk;    // samples whose walk is left to it (distance known)
   unsigned long long nmigrate; // searches that outgrew the small table
-  unsigned long long nbig;     // warp searches handed on to the CTA launch
-  unsigned long long bignext;  // next of them for the CTA launch
   int err;
   int pad;
 };
+// Where the searches by CTAs of a job start (bidir_log.cuh; each hands on to
+// the next what outgrows it): small or wide CTAs with their state in shared
+// memory, or the tables in global memory.
+constexpr int64_t kBidirQueue = (int64_t)1 << 16;  // default queue entries per ball or cone side
+constexpr int kTierSmall = 0, kTierWide = 1, kTierGlobal = 2;
 struct BiWS {
   DevBuf tab1, tab2, lists, sig, epochs, ctl, aoff, dsearch, dwalk, arena;
   DevBuf tabw, epw;        // warp searches: node tables and epochs (none when WQ = 0)
-  DevBuf big;              // ids the warp searches hand on to the CTA searches
+  DevBuf big, far;         // ids that a launch hands on to the next (used in turn)
+  int tier = 0;            // where searches by CTAs start (kTier*)
   int nslots = 0;
   int64_t QC = 0;
   int64_t H1 = 0;
@@ -150,7 +155,7 @@ struct cen_job {
   std::unique_ptr<cen::BiWS> bws;
   int sampler = 0;                          // 0 bidirectional (bit-parallel for what it defers), 1 bit-parallel
   size_t bidir_budget = (size_t)16 << 30;   // bytes of per-slot workspace
-  int64_t bidir_queue = (int64_t)1 << 16;   // entries per ball / cone list
+  int64_t bidir_queue = cen::kBidirQueue;   // entries per ball / cone list
   int64_t bidir_table = -1;                 // small-table entries per CTA (-1: sized for L2, 0: none)
   int bidir_warps = -1;  // 1: warp searches, what they hand on by CTAs; 0: CTAs only; -1: by the graph's record
   uint64_t bidir_deferred_search = 0;       // samples it left whole to the bit-parallel sampler
@@ -165,10 +170,12 @@ struct cen_job {
 
 namespace cen {
 void sample_append(cen_job *job, uint64_t m_new);
-void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap);
+void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages);
+void bidir_launch_rest(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages, uint64_t left);
 // Entries of each list of a warp search for a CTA queue of QC entries (0: warp searches off).
 int64_t bidir_warp_queue(int64_t QC);
 size_t bidir_warp_bytes_per_slot();
+bool bidir_shared_ok(int32_t n);
 // E[d^2] / E[d] of the graph's degrees (out and in, the larger), computed once.
 double graph_branching(const cen_graph *g, cudaStream_t st);
 // The bit-parallel sampler's chunk tables of the graph's long out- and in-rows

@@ -168,6 +168,19 @@ int resident_grid(const void *kernel, int block) {
   return g;
 }
 
+void allow_shared(const void *kernel, size_t bytes) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void *>, size_t> done;
+  int dev = 0;
+  CEN_CK(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(mu);
+  size_t &have = done[{dev, kernel}];
+  if (have >= bytes) return;
+  CEN_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  CEN_CK(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+  have = bytes;
+}
+
 // -------------------------------------------------------------- scans
 constexpr int kScanThreads = 1024, kScanItems = 4, kScanTile = kScanThreads * kScanItems;
 

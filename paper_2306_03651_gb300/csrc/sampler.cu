@@ -1286,8 +1286,11 @@ int64_t offsets_from_distances(cen_job *job, uint64_t m0, uint64_t m_new, int64_
 // one).  The small tables are sized so that all of them take about kTableL2
 // bytes (they stay in L2), unless a size was set.
 constexpr size_t kTableL2 = (size_t)80 << 20;
-// Measured: warp searches are 1.3-1.75x faster than whole-CTA searches on BA graphs and small
-// R-MATs (E[d^2]/E[d] from 19 to 126) and slower on R-MAT 16, 18 and directed 22 (684 to 2,244).
+// Measured with the tables in global memory: warp searches are 1.3-1.75x faster than whole-CTA
+// searches on BA graphs and small R-MATs (E[d^2]/E[d] from 19 to 126) and slower on R-MAT 16, 18
+// and directed 22 (684 to 2,244).  CTA searches in shared memory are faster than warp searches on
+// all of them (65,536 pairs: BA n = 2,000 0.67 against 1.44 ms, BA n = 400,000 2.56 against 4.65,
+// R-MAT 12 0.69 against 1.36).
 constexpr double kWarpBranching = 256.0;
 
 void bidir_setup(cen_job *job, uint64_t m_new) {
@@ -1296,10 +1299,12 @@ void bidir_setup(cen_job *job, uint64_t m_new) {
   const int64_t QC = std::max<int64_t>(16, std::min<int64_t>(n, job->bidir_queue));
   int64_t H2 = 1024;
   while (H2 < 4 * QC) H2 *= 2;
-  // by default, warp searches only where frontiers grow slowly (E[d^2] / E[d], the mean degree at
-  // the far end of an arc, at most kWarpBranching), and until a call hands too many on
+  // searches start in shared memory unless a table size was set or the ids are too long for it
+  const int tier = job->bidir_table < 0 && bidir_shared_ok(n) ? job->g->bidir_tier.load() : kTierGlobal;
+  // by default, warp searches only where that does not hold and frontiers grow slowly (E[d^2] / E[d],
+  // the mean degree at the far end of an arc, at most kWarpBranching), and until a call hands too many on
   const bool warps = job->bidir_warps > 0 ||
-                     (job->bidir_warps < 0 && !job->g->bidir_warps_off.load() &&
+                     (job->bidir_warps < 0 && tier == kTierGlobal && !job->g->bidir_warps_off.load() &&
                       graph_branching(job->g, st) <= kWarpBranching);
   const int64_t WQ = warps ? bidir_warp_queue(QC) : 0;
   auto per_slot = [&](int64_t h1) {
@@ -1308,7 +1313,7 @@ void bidir_setup(cen_job *job, uint64_t m_new) {
   const size_t res = (size_t)bidir_resident_slots();
   int slots = (int)std::min<size_t>(res, std::max<size_t>(1, job->bidir_budget / per_slot(0)));
   int64_t H1 = 0;
-  if (job->bidir_table < 0 && !job->g->bidir_table_off.load()) {
+  if (job->bidir_table < 0 && tier == kTierGlobal && !job->g->bidir_table_off.load()) {
     H1 = 1024;
     while ((size_t)(2 * H1) * 8 * (size_t)slots <= kTableL2 && 2 * H1 < H2) H1 *= 2;
   } else if (job->bidir_table > 0) {
@@ -1353,8 +1358,10 @@ void bidir_setup(cen_job *job, uint64_t m_new) {
     wk.dev = dev;
   }
   for (DevBuf *b : {&wk.tab1, &wk.tab2, &wk.lists, &wk.sig, &wk.epochs, &wk.tabw, &wk.epw}) b->st = st;
+  wk.tier = tier;
   wk.ctl.ensure(sizeof(BiCtl), st);
   wk.big.ensure(8 * (size_t)m_new, st);
+  wk.far.ensure(8 * (size_t)m_new, st);
   wk.aoff.ensure(8 * (size_t)m_new, st);
   wk.dsearch.ensure(8 * (size_t)m_new, st);
   wk.dwalk.ensure(8 * (size_t)m_new, st);
@@ -1371,6 +1378,17 @@ static BiCtl bidir_finish(cen_job *job) {
   return h;
 }
 
+// The searches of one call, to their end; *stages launches' counts are in the
+// result.
+static BiCtl bidir_search(cen_job *job, uint64_t m0, uint64_t m_new, int64_t cap, int *stages) {
+  bidir_launch(job, m0, m_new, cap, stages);
+  BiCtl h = bidir_finish(job);
+  const uint64_t left = h.nout[*stages - 1];
+  if (!left) return h;
+  bidir_launch_rest(job, m0, m_new, cap, stages, left);
+  return bidir_finish(job);
+}
+
 // Bidirectional form: one CTA per sample writes its members to an arena;
 // what it defers runs on the bit-parallel sampler (see bidir.cu).  Returns
 // the new members.
@@ -1381,8 +1399,8 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   const double mean = job->m ? (double)job->members / (double)job->m : 4.0;
   int64_t cap = (int64_t)((double)m_new * std::max(8.0, 2.0 * mean)) + ((int64_t)1 << 20);
   bw.arena.ensure(4 * (size_t)cap, st);
-  bidir_launch(job, m0, m_new, cap);
-  BiCtl h = bidir_finish(job);
+  int stages = 0;
+  BiCtl h = bidir_search(job, m0, m_new, cap, &stages);
   if ((int64_t)h.cursor > cap) {
     // The arena was short (long paths in a job's first round, where no mean
     // is known yet): the cursor has counted every walk's members, so size the
@@ -1390,12 +1408,23 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
     // instead of leaving those walks to the bit-parallel sampler.
     cap = (int64_t)h.cursor + ((int64_t)1 << 20);
     bw.arena.ensure(4 * (size_t)cap, st);
-    bidir_launch(job, m0, m_new, cap);
-    h = bidir_finish(job);
+    h = bidir_search(job, m0, m_new, cap, &stages);
   }
   if (job->bidir_table < 0 && m_new >= 1024 && 2 * h.nmigrate > m_new) job->g->bidir_table_off.store(true);
   // warp searches pay off when few outgrow a warp; each one handed on is searched twice
-  if (job->bidir_warps < 0 && bw.WQ && m_new >= 1024 && 10 * h.nbig > 3 * m_new) job->g->bidir_warps_off.store(true);
+  const unsigned long long nbig = bw.WQ ? h.nout[0] : 0;
+  // a size of search that handed on most of many samples is left out from now on (not when a
+  // short queue made it)
+  if (bw.tier != kTierGlobal && job->bidir_queue >= kBidirQueue) {
+    int tier = bw.tier;
+    for (int k = bw.WQ ? 1 : 0; tier < kTierGlobal && k < stages; ++k, ++tier) {
+      const unsigned long long in = k ? h.nout[k - 1] : m_new;
+      if (in < 512 || 2 * h.nout[k] <= in) break;
+    }
+    if (tier > bw.tier) job->g->bidir_tier.store(tier);
+    if (tier == kTierGlobal) job->g->bidir_warps_off.store(true);  // such searches outgrow a warp too
+  }
+  if (job->bidir_warps < 0 && bw.WQ && m_new >= 1024 && 10 * nbig > 3 * m_new) job->g->bidir_warps_off.store(true);
   std::vector<uint64_t> search(h.nsearch), walk(h.nwalk);
   if (h.nsearch)
     CEN_CK(cudaMemcpyAsync(search.data(), bw.dsearch.p, 8 * h.nsearch, cudaMemcpyDeviceToHost, st));
@@ -1445,7 +1474,7 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   job->bidir_deferred_search += h.nsearch;
   job->bidir_deferred_walk += walk.size();
   job->bidir_migrated += h.nmigrate;
-  job->bidir_escalated += h.nbig;
+  job->bidir_escalated += nbig;
   return total;
 }
 
