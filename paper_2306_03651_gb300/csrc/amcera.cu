@@ -5,49 +5,151 @@
 // sum_{u in S} R_q^u is the sum of the <= k largest positive R_q^u (the
 // objective is additive in S), found per row by an exact MSB-first radix
 // select; the same select over c_u gives the wimpy-variance numerator.
+#include <algorithm>
+#include <cstddef>
+#include <cstring>
 #include <mutex>
 
-#include "job.cuh"
+#include "heavy.cuh"
 
 namespace cen {
 
-// Warp per node u with c_u > 0: lanes take 32 incident samples at a time; for
-// each sign word the warp ballots bit q across the 32 samples (the word's
-// rows only) and lane q adds the popcount.  The block sums its scanned
-// incidences before one atomic.
-__global__ void __launch_bounds__(256) k_rade(int32_t n, int t, int nw, const int64_t *__restrict__ noff,
+// ---- R over incidence rows
+// A warp takes one chunk (at most kRadeChunk incidences) of one listed node's
+// row.  Each lane adds the sign words of its incidences into bit-sliced
+// counters (plane b holds bit b of 32 column counts), so that an incidence
+// costs a load and a few logic operations for 32 sign vectors instead of a
+// ballot for each.  Five butterfly steps add the lanes' counters, bit-sliced
+// too, and lane q reads column q.  A node with more than one chunk adds its
+// parts into R, which starts at zero.  Bound by the gathered sign rows and, for
+// short rows, by the butterfly.  R-MAT 16, m = 262,144, t = 256: 4.6 ms (a warp
+// per node of any row length, ballots) -> 0.06; R-MAT 18, m = 65,536, t = 10:
+// 0.074 -> 0.018 ms.
+template <int NB>
+__device__ __forceinline__ void planes_add(uint32_t *p, uint32_t x) {  // one bit per column
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const uint32_t carry = p[b] & x;
+    p[b] ^= x;
+    x = carry;
+  }
+}
+// Adds NB-plane counters over the warp's lanes; column q's total in lane q.
+template <int NB>
+__device__ __forceinline__ int32_t planes_total(const uint32_t *in) {
+  const int lane = threadIdx.x & 31;
+  uint32_t p[NB + 5];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) p[b] = in[b];
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    uint32_t carry = 0;
+#pragma unroll
+    for (int b = 0; b < NB + s; ++b) {
+      const uint32_t y = __shfl_xor_sync(0xffffffffu, p[b], 1 << s);
+      const uint32_t half = p[b] ^ y;
+      const uint32_t up = (p[b] & y) | (half & carry);
+      p[b] = half ^ carry;
+      carry = up;
+    }
+    p[NB + s] = carry;
+  }
+  int32_t v = 0;
+#pragma unroll
+  for (int b = 0; b < NB + 5; ++b) v |= (int32_t)((p[b] >> lane) & 1u) << b;
+  return v;
+}
+
+constexpr int kRadePlanes = 7;  // a lane's share of a chunk: at most 64 incidences
+static_assert(kRadeChunk / 32 < (1 << kRadePlanes), "a lane's counters hold its share of a chunk");
+
+// One chunk's column sums for words w0 .. w0 + W - 1 of the sign rows.
+template <int W, int NB, bool VEC>
+__device__ __forceinline__ void rade_words(const int32_t *__restrict__ samp, int len, int nw, int w0, int t,
+                                           const uint32_t *__restrict__ sign, int32_t *R, int64_t stride, int64_t at,
+                                           bool add) {
+  const int lane = threadIdx.x & 31;
+  uint32_t p[W][NB];
+#pragma unroll
+  for (int w = 0; w < W; ++w)
+#pragma unroll
+    for (int b = 0; b < NB; ++b) p[w][b] = 0;
+#pragma unroll 2
+  for (int i = lane; i < len; i += 32) {
+    const uint32_t *row = sign + (int64_t)samp[i] * nw + w0;
+    if constexpr (VEC) {
+      const uint4 x = *(const uint4 *)row;
+      planes_add<NB>(p[0], x.x);
+      planes_add<NB>(p[1], x.y);
+      planes_add<NB>(p[2], x.z);
+      planes_add<NB>(p[3], x.w);
+    } else {
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        if (w0 + w < nw) planes_add<NB>(p[w], row[w]);
+    }
+  }
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    if (w0 + w >= nw) break;
+    const int32_t v = 2 * planes_total<NB>(p[w]) - len;
+    const int q = 32 * (w0 + w) + lane;
+    if (q >= t) continue;
+    int32_t *dst = R + (int64_t)q * stride + at;
+    if (add)
+      atomicAdd(dst, v);
+    else
+      *dst = v;
+  }
+}
+
+template <int W, bool VEC>
+__global__ void __launch_bounds__(256) k_rade(HeavyView H, int t, int nw, const int64_t *__restrict__ noff,
                                               const int32_t *__restrict__ nsamp, const uint32_t *__restrict__ sign,
-                                              int32_t *R, unsigned long long *units) {
+                                              int32_t *R, int64_t stride, unsigned long long *units) {
+  const uint32_t nwarps = gridDim.x * 8, nchunks = H.ctl->nchunks;
+  unsigned long long scanned = 0;
+  for (uint32_t ci = blockIdx.x * 8 + (threadIdx.x >> 5); ci < nchunks; ci += nwarps) {
+    const uint2 ch = H.chunks[ci];
+    const int32_t u = H.list[ch.x], cu = H.c[ch.x];
+    const int first = (int)ch.y * kRadeChunk, len = min(kRadeChunk, cu - first);
+    const int32_t *samp = nsamp + noff[u] + first;
+    const bool add = cu > kRadeChunk;
+    for (int w0 = 0; w0 < nw; w0 += W) {
+      if (len <= 32)
+        rade_words<W, 1, VEC>(samp, len, nw, w0, t, sign, R, stride, ch.x, add);
+      else if (len <= 32 * 7)
+        rade_words<W, 3, VEC>(samp, len, nw, w0, t, sign, R, stride, ch.x, add);
+      else
+        rade_words<W, kRadePlanes, VEC>(samp, len, nw, w0, t, sign, R, stride, ch.x, add);
+    }
+    scanned += (unsigned long long)len;
+  }
   __shared__ unsigned long long s_scanned;
   if (threadIdx.x == 0) s_scanned = 0;
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  unsigned long long scanned = 0;
-  for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += nwarps) {
-    const int64_t r0 = noff[u], r1 = noff[u + 1];
-    const int32_t cu = (int32_t)(r1 - r0);
-    if (cu == 0) continue;  // R rows are zero-filled
-    for (int w = 0; w < nw; ++w) {
-      const int qn = min(32, t - 32 * w);  // rows of this word
-      int32_t P = 0;
-      for (int64_t base = r0; base < r1; base += 32) {
-        const int64_t i = base + lane;
-        const uint32_t x = i < r1 ? sign[(int64_t)nsamp[i] * nw + w] : 0u;
-#pragma unroll 8
-        for (int q = 0; q < qn; ++q) {
-          const int c = __popc(__ballot_sync(0xffffffffu, (x >> q) & 1u));
-          if (lane == q) P += c;
-        }
-      }
-      const int q = 32 * w + lane;
-      if (q < t) R[(int64_t)q * n + u] = 2 * P - cu;
-    }
-    scanned += (unsigned long long)cu;
-  }
-  if (lane == 0 && scanned) atomicAdd(&s_scanned, scanned);
+  if ((threadIdx.x & 31) == 0 && scanned) atomicAdd(&s_scanned, scanned);
   __syncthreads();
   if (threadIdx.x == 0 && s_scanned) atomicAdd(units, s_scanned);
+}
+
+// Enqueues R (t rows at `stride`, column = list entry) of H's nodes.
+static void rade_enqueue(cen_job *job, const HeavyView &H, int32_t *R, int64_t stride, cudaStream_t run) {
+  const int t = job->t, nw = job->nw;
+  CEN_CK(cudaMemsetAsync(R, 0, 4 * (size_t)stride * t, run));
+  unsigned long long *units = (unsigned long long *)(job->stats.d_units + K_RADE);
+  const int grid = sm_count() * 8;
+  const int64_t *noff = job->noff.as<int64_t>();
+  const int32_t *nsamp = job->nsamp.as<int32_t>();
+  const uint32_t *sign = job->sign.as<uint32_t>();
+  launch(&job->stats, K_RADE, run, [&] {
+    if (nw == 1)
+      k_rade<1, false><<<grid, 256, 0, run>>>(H, t, nw, noff, nsamp, sign, R, stride, units);
+    else if (nw % 4 == 0 && ((uintptr_t)sign & 15) == 0)  // 16-byte sign loads are aligned
+      k_rade<4, true><<<grid, 256, 0, run>>>(H, t, nw, noff, nsamp, sign, R, stride, units);
+    else
+      k_rade<4, false><<<grid, 256, 0, run>>>(H, t, nw, noff, nsamp, sign, R, stride, units);
+  });
 }
 
 // ------------------------------------------------------------ radix select
@@ -155,6 +257,91 @@ __global__ void __launch_bounds__(256) k_sel_step(int nrows, int shift, SelRow *
   rows[r] = out;
 }
 
+// ---- top-k over the heavy nodes
+// A block per row with the row's values in registers: the k-th largest
+// positive value by bisection, then the sum.  done = 1 when no unlisted node
+// (whose values are below tau) could raise the sum: fewer than k positive
+// values need every touched node listed (tau = 1), else the k-th must be at
+// least tau - 1.  One launch of some 8 us (barriers of the bisection) in place
+// of two per digit: R-MAT 18 0.08 -> 0.008 ms; directed R-MAT 22, t = 100, whose
+// rows of 4.2 million were read three times: 1.9 -> 0.008 ms.
+constexpr int kTopThreads = 1024, kTopPer = kHeavyMax / kTopThreads;
+__global__ void __launch_bounds__(kTopThreads) k_heavy_top(HeavyView H, const int32_t *__restrict__ R, int64_t stride,
+                                                           int t, int32_t k, SelRow *rows) {
+  __shared__ uint32_t s_cnt[2][32];
+  __shared__ unsigned long long s_sum[32];
+  const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int32_t count = (int32_t)H.ctl->count, tau = H.ctl->tau;
+  const int32_t *row = r < t ? R + (int64_t)r * stride : H.c;
+  int32_t v[kTopPer];
+  uint32_t most = 0, npos = 0;
+#pragma unroll
+  for (int i = 0; i < kTopPer; ++i) {
+    const int at = i * kTopThreads + tid;
+    v[i] = at < count ? max(row[at], 0) : 0;
+    most = max(most, (uint32_t)v[i]);
+    npos += v[i] > 0;
+  }
+  most = __reduce_max_sync(0xffffffffu, most);
+  npos = __reduce_add_sync(0xffffffffu, npos);
+  if (lane == 0) {
+    s_cnt[0][wid] = most;
+    s_cnt[1][wid] = npos;
+  }
+  __syncthreads();
+  most = __reduce_max_sync(0xffffffffu, s_cnt[0][lane]);
+  npos = __reduce_add_sync(0xffffffffu, s_cnt[1][lane]);
+  uint32_t kth = 0, above = npos;  // values > kth (kth = 0: every positive value is in)
+  if (npos >= (uint32_t)k) {
+    uint32_t lo = 1, hi = most;  // the largest value that at least k values reach
+    int par = 0;
+    while (lo < hi) {
+      const uint32_t mid = lo + ((hi - lo + 1) >> 1);
+      uint32_t c = 0;
+#pragma unroll
+      for (int i = 0; i < kTopPer; ++i) c += (uint32_t)v[i] >= mid;
+      c = __reduce_add_sync(0xffffffffu, c);
+      __syncthreads();  // the last turn's counts have been read
+      if (lane == 0) s_cnt[par][wid] = c;
+      __syncthreads();
+      c = __reduce_add_sync(0xffffffffu, s_cnt[par][lane]);
+      par ^= 1;
+      if (c >= (uint32_t)k)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    kth = lo;
+  }
+  unsigned long long sum = 0;
+  uint32_t c = 0;
+#pragma unroll
+  for (int i = 0; i < kTopPer; ++i)
+    if ((uint32_t)v[i] > kth) {
+      sum += (unsigned long long)v[i];
+      ++c;
+    }
+  sum = warp_sum(sum);
+  c = __reduce_add_sync(0xffffffffu, c);
+  __syncthreads();
+  if (lane == 0) {
+    s_sum[wid] = sum;
+    s_cnt[0][wid] = c;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    sum = 0;
+    above = 0;
+    for (int w = 0; w < 32; ++w) {
+      sum += s_sum[w];
+      above += s_cnt[0][w];
+    }
+    if (kth) sum += (unsigned long long)(k - (int32_t)above) * kth;
+    rows[r].sum = (long long)sum;
+    rows[r].done = tau <= 1 || (kth != 0 && (int32_t)kth >= tau - 1);
+  }
+}
+
 // Enqueues on `run` the sums of the <= k largest positive entries of each of
 // `nrows` rows of length n (select state sized beforehand, see mcera_prepare);
 // the per-row results reach hdst (pinned, nrows SelRow) once `run` drains.
@@ -183,49 +370,109 @@ static void topk_enqueue(cen_job *job, const int32_t *vals, int64_t n, int nrows
 // Host bytes mcera_enqueue copies into: t + 1 select rows, then b_H.
 size_t mcera_result_bytes(const cen_job *job) { return sizeof(SelRow) * (size_t)(job->t + 1) + 8; }
 
+// The list that k_rade takes for R over all nodes (column = node): every node
+// with its c_u, and the chunks of every row.  The incidence must be current.
+static HeavyView all_nodes(cen_job *job, cudaStream_t st) {
+  const int32_t n = job->g->n;
+  HeavyCtl *ctl = job->hctl_all.as<HeavyCtl>();
+  CEN_CK(cudaMemsetAsync(ctl, 0, offsetof(HeavyCtl, hist), st));
+  launch(&job->stats, K_RADE, st, [&] {
+    heavy_list_all(job->c.as<int32_t>(), n, ctl, job->hlist_all.as<int32_t>(), job->hc_all.as<int32_t>(),
+                   job->hchunks_all.as<uint2>(), st);
+  });
+  return HeavyView{ctl, job->hlist_all.as<int32_t>(), job->hc_all.as<int32_t>(),
+                   job->hchunks_all.as<uint2>()};
+}
+
+// Sizes the workspace of R over all nodes (allocations ordered on the job's stream).
+static void rade_all_prepare(cen_job *job) {
+  cudaStream_t st = job->st;
+  const size_t n = (size_t)job->g->n;
+  job->R.ensure(4 * n * (job->t + 1), st);
+  job->hctl_all.ensure(sizeof(HeavyCtl), st);
+  job->hlist_all.ensure(4 * n, st);
+  job->hc_all.ensure(4 * n, st);
+  job->hchunks_all.ensure(8 * (n + (size_t)job->members / kRadeChunk + 1), st);
+}
+
+// R over all nodes into job->R (row t: c), on `run`.
+void rade_all(cen_job *job, cudaStream_t run) {
+  const int32_t n = job->g->n;
+  rade_enqueue(job, all_nodes(job, run), job->R.as<int32_t>(), n, run);
+  CEN_CK(cudaMemcpyAsync(job->R.as<int32_t>() + (size_t)n * job->t, job->c.p, 4 * (size_t)n, cudaMemcpyDeviceToDevice,
+                         run));
+  job->rade_all_m = job->m;
+}
+
+// R over all nodes for cen_job_copy_rade, when the AMCERA did not need it.
+void rade_for_copy(cen_job *job) {
+  if (job->rade_all_m == job->m) return;
+  rade_all_prepare(job);
+  rade_all(job, job->st);
+}
+
 // Sizes the AMCERA workspace (allocations ordered on the job's stream).  The
-// incidence must be current.
+// incidence must be current, and the heavy nodes listed.
 void mcera_prepare(cen_job *job, int32_t k) {
   CEN_REQUIRE(k >= 1, CEN_EINVAL, "cen_mcera: k must be >= 1");
   cudaStream_t st = job->st;
   const int nrows = job->t + 1;
-  job->R.ensure(4 * (size_t)job->g->n * nrows, st);
   job->selst.ensure(sizeof(SelRow) * (size_t)nrows, st);
+  if (!job->rade_all) {
+    job->Rh.ensure(4 * (size_t)std::min(job->g->n, kHeavyMax) * job->t, st);
+    return;
+  }
+  rade_all_prepare(job);
   job->selh.ensure((size_t)nrows * 256 * (4 + 8), st);
 }
 
-// Enqueues the AMCERA of Alg. 1 on stream `run` (after mcera_prepare): rows
-// 0 .. t-1 of R are R_q^u, row t is c_u, so one selection gives every Rnum and
-// Wnum.  Results reach hdst (pinned, mcera_result_bytes) once `run` drains.
-void mcera_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst) {
-  Stats *S = &job->stats;
+// Enqueues the AMCERA of Alg. 1 on stream `run` (after mcera_prepare): every
+// Rnum (rows 0 .. t-1) and Wnum (row t, over c_u), over the heavy nodes or over
+// all.  Results reach hdst (pinned, mcera_result_bytes) once `run` drains.
+void mcera_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool heavy) {
   const int32_t n = job->g->n;
   const int t = job->t;
-  CEN_CK(cudaMemsetAsync(job->R.p, 0, 4 * (size_t)n * t, run));
-  launch(S, K_RADE, run, [&] {
-    k_rade<<<grid_for((size_t)n * 32, 256, sm_count() * 64), 256, 0, run>>>(n, t, job->nw, job->noff.as<int64_t>(),
-                                                                       job->nsamp.as<int32_t>(),
-                                                                       job->sign.as<uint32_t>(), job->R.as<int32_t>(),
-                                                                       (unsigned long long *)(job->stats.d_units + K_RADE));
-  });
-  CEN_CK(cudaMemcpyAsync(job->R.as<int32_t>() + (size_t)n * t, job->c.p, 4 * (size_t)n, cudaMemcpyDeviceToDevice,
-                         run));
   SelRow *hrows = (SelRow *)hdst;
-  // |R_q^u| <= c_u <= m: every value the select ranks is at most m
-  topk_enqueue(job, job->R.as<int32_t>(), n, t + 1, k, run, hrows, (int64_t)job->m);
+  if (heavy) {
+    const HeavyView H = heavy_view(job);
+    const int64_t stride = std::min(n, kHeavyMax);
+    SelRow *rows = job->selst.as<SelRow>();
+    rade_enqueue(job, H, job->Rh.as<int32_t>(), stride, run);
+    launch(&job->stats, K_SELECT, run, [&] {
+      k_heavy_top<<<t + 1, kTopThreads, 0, run>>>(H, job->Rh.as<int32_t>(), stride, t, k, rows);
+    });
+    CEN_CK(cudaMemcpyAsync(hrows, rows, sizeof(SelRow) * (size_t)(t + 1), cudaMemcpyDeviceToHost, run));
+  } else {
+    rade_all(job, run);
+    // |R_q^u| <= c_u <= m: every value the select ranks is at most m
+    topk_enqueue(job, job->R.as<int32_t>(), n, t + 1, k, run, hrows, (int64_t)job->m);
+  }
   if (job->m) CEN_CK(cudaMemcpyAsync(hrows + t + 1, job->bmax.p, 4, cudaMemcpyDeviceToHost, run));  // b_H = 0 if m = 0
 }
 
-// Rnum[t], Wnum and b_H from the copied result.
-void mcera_result(cen_job *job, int32_t k, const void *h, int64_t *Rnum, int64_t *Wnum, int32_t *b) {
+// Rnum[t], Wnum and b_H from the copied result; false when the heavy nodes did
+// not decide every row.
+bool mcera_result(cen_job *job, int32_t k, const void *h, int64_t *Rnum, int64_t *Wnum, int32_t *b) {
   const SelRow *hrows = (const SelRow *)h;
   const int t = job->t;
+  for (int q = 0; q <= t; ++q)
+    if (!hrows[q].done) return false;
   for (int q = 0; q < t; ++q) Rnum[q] = hrows[q].sum;
   *Wnum = hrows[t].sum;  // the c_u are positive, so this is the sum of the k largest
   int hb = 0;
   memcpy(&hb, hrows + t + 1, 4);
   *b = job->m ? hb : 0;
   job->rade_valid_k = k;
+  return true;
+}
+
+// The AMCERA over all nodes, on the job's stream.
+static void mcera_over_all(cen_job *job, int32_t k, void *h, int64_t *Rnum, int64_t *Wnum, int32_t *b) {
+  job->rade_all = true;  // the job's later samples spread over as many nodes
+  mcera_prepare(job, k);
+  mcera_enqueue(job, k, job->st, h, false);
+  CEN_CK(cudaStreamSynchronize(job->st));
+  CEN_REQUIRE(mcera_result(job, k, h, Rnum, Wnum, b), CEN_ECUDA, "cen_mcera: the select left a row open");
 }
 
 // greedyCover on the job's stream and the AMCERA on its second stream at the
@@ -236,6 +483,7 @@ void cover_and_mcera(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint6
   CEN_REQUIRE(k >= 1, CEN_EINVAL, "cen_cover_and_mcera: k must be >= 1");
   Range range("cen_cover_and_mcera");
   build_incidence(job);
+  build_heavy(job);
   greedy_prepare(job, k);
   mcera_prepare(job, k);
   const size_t gb = (greedy_result_bytes(k) + 15) & ~(size_t)15;
@@ -243,9 +491,9 @@ void cover_and_mcera(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint6
   job->aux.ensure();
   CEN_CK(cudaEventRecord(job->aux.fork, job->st));
   CEN_CK(cudaStreamWaitEvent(job->aux.st, job->aux.fork, 0));
-  greedy_enqueue(job, k, job->st, h);
+  greedy_enqueue(job, k, job->st, h, !job->greedy_all);
   try {
-    mcera_enqueue(job, k, job->aux.st, h + gb);
+    mcera_enqueue(job, k, job->aux.st, h + gb, !job->rade_all);
   } catch (...) {  // still join, so that nothing on the job's stream outruns the second stream
     cudaEventRecord(job->aux.join, job->aux.st);
     cudaStreamWaitEvent(job->st, job->aux.join, 0);
@@ -254,8 +502,8 @@ void cover_and_mcera(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint6
   CEN_CK(cudaEventRecord(job->aux.join, job->aux.st));
   CEN_CK(cudaStreamWaitEvent(job->st, job->aux.join, 0));
   CEN_CK(cudaStreamSynchronize(job->st));
-  greedy_result(h, S, S_size, covered);
-  mcera_result(job, k, h + gb, Rnum, Wnum, b);
+  if (!greedy_result(h, S, S_size, covered)) greedy_over_all(job, k, h, S, S_size, covered);
+  if (!mcera_result(job, k, h + gb, Rnum, Wnum, b)) mcera_over_all(job, k, h + gb, Rnum, Wnum, b);
 }
 
 // ----------------------------------------------- AMCERA of a split sample
@@ -264,18 +512,11 @@ void cover_and_mcera(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint6
 // (R and c are sums over samples) and takes shard_topk of the sum.
 void shard_rade(cen_job *job, int32_t *R_out, int32_t *b) {
   build_incidence(job);
-  mcera_prepare(job, 1);
+  rade_all_prepare(job);
   cudaStream_t st = job->st;
   const int32_t n = job->g->n;
-  const int t = job->t;
-  CEN_CK(cudaMemsetAsync(job->R.p, 0, 4 * (size_t)n * t, st));
-  launch(&job->stats, K_RADE, st, [&] {
-    k_rade<<<grid_for((size_t)n * 32, 256, sm_count() * 64), 256, 0, st>>>(
-        n, t, job->nw, job->noff.as<int64_t>(), job->nsamp.as<int32_t>(), job->sign.as<uint32_t>(),
-        job->R.as<int32_t>(), (unsigned long long *)(job->stats.d_units + K_RADE));
-  });
-  CEN_CK(cudaMemcpyAsync(job->R.as<int32_t>() + (size_t)n * t, job->c.p, 4 * (size_t)n, cudaMemcpyDeviceToDevice, st));
-  CEN_CK(cudaMemcpyAsync(R_out, job->R.p, 4 * (size_t)n * (t + 1), cudaMemcpyDeviceToDevice, st));
+  rade_all(job, st);
+  CEN_CK(cudaMemcpyAsync(R_out, job->R.p, 4 * (size_t)n * (job->t + 1), cudaMemcpyDeviceToDevice, st));
   int32_t *h = (int32_t *)host_staging(job, 4);
   *h = 0;
   if (job->m) CEN_CK(cudaMemcpyAsync(h, job->bmax.p, 4, cudaMemcpyDeviceToHost, st));
@@ -300,11 +541,12 @@ void mcera(cen_job *job, int32_t k, int64_t *Rnum, int64_t *Wnum, int32_t *b) {
   CEN_REQUIRE(k >= 1, CEN_EINVAL, "cen_mcera: k must be >= 1");
   Range range("cen_mcera");
   build_incidence(job);
+  build_heavy(job);
   mcera_prepare(job, k);
   void *h = host_staging(job, mcera_result_bytes(job));
-  mcera_enqueue(job, k, job->st, h);
+  mcera_enqueue(job, k, job->st, h, !job->rade_all);
   CEN_CK(cudaStreamSynchronize(job->st));
-  mcera_result(job, k, h, Rnum, Wnum, b);
+  if (!mcera_result(job, k, h, Rnum, Wnum, b)) mcera_over_all(job, k, h, Rnum, Wnum, b);
 }
 
 }  // namespace cen

@@ -1,10 +1,13 @@
 // Node -> sample incidence and greedyCover(k, H) (Sec. 3.1; Alg. 1 line "greedyCover").
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <cstddef>
 #include <cstdlib>
+#include <map>
 #include <mutex>
 
-#include "job.cuh"
+#include "heavy.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -55,6 +58,154 @@ void build_incidence(cen_job *job) {
   job->inc_m = job->m;
 }
 
+// ------------------------------------------------------- heavy nodes
+// Counts of the c_u buckets.
+__global__ void __launch_bounds__(256) k_heavy_hist(const int32_t *__restrict__ c, int32_t n, HeavyCtl *ctl) {
+  __shared__ uint32_t h[kHeavyBuckets];
+  for (int i = threadIdx.x; i < kHeavyBuckets; i += 256) h[i] = 0;
+  __syncthreads();
+  for (int64_t u = (int64_t)blockIdx.x * 256 + threadIdx.x; u < n; u += (int64_t)gridDim.x * 256) {
+    const int32_t cu = c[u];
+    if (cu > 0) atomicAdd(&h[heavy_bucket((uint32_t)cu)], 1u);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kHeavyBuckets; i += 256)
+    if (h[i]) atomicAdd(&ctl->hist[i], h[i]);
+}
+
+// Lists the nodes with c_u >= tau (tau from the bucket counts, by every block;
+// order of arrival) with their c_u, the chunks of their rows, and for every
+// node its list entry or -1.  With `all`, entry u is node u and tau is 1.
+__global__ void __launch_bounds__(256) k_heavy_list(const int32_t *__restrict__ c, int32_t n, bool all, HeavyCtl *ctl,
+                                                    int32_t *list, int32_t *hc, int32_t *idx, uint2 *chunks) {
+  __shared__ uint32_t wsum[8];
+  __shared__ int s_cut;
+  const int tid = threadIdx.x, lane = tid & 31;
+  uint32_t tau = 1;
+  if (!all) {
+    // thread i holds buckets from the top: [B - (i+1) P, B - i P)
+    constexpr int P = (kHeavyBuckets + 255) / 256;
+    const int top = kHeavyBuckets - tid * P;
+    uint32_t sum = 0;
+    for (int q = 0; q < P; ++q)
+      if (top - 1 - q >= 1) sum += ctl->hist[top - 1 - q];
+    uint32_t inc = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[tid >> 5] = inc;
+    if (tid == 0) s_cut = 1;  // every bucket fits
+    __syncthreads();
+    for (int w = 0; w < (tid >> 5); ++w) inc += wsum[w];
+    if (inc > (uint32_t)kHeavyMax && inc - sum <= (uint32_t)kHeavyMax) {  // the bucket that overflows is in here
+      uint32_t run = inc - sum;
+      for (int q = 0; q < P && top - 1 - q >= 1; ++q) {
+        run += ctl->hist[top - 1 - q];
+        if (run > (uint32_t)kHeavyMax) {
+          s_cut = top - q;  // the buckets above it
+          break;
+        }
+      }
+    }
+    __syncthreads();
+    tau = s_cut >= kHeavyBuckets ? 0x7fffffffu : heavy_bucket_low(s_cut);
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    ctl->tau = (int32_t)tau;
+    if (all) ctl->count = (uint32_t)n;
+  }
+  const int64_t span = ((int64_t)n + 31) & ~(int64_t)31;  // whole warps
+  for (int64_t u = (int64_t)blockIdx.x * 256 + tid; u < span; u += (int64_t)gridDim.x * 256) {
+    const int32_t cu = u < n ? c[u] : 0;
+    const bool in = cu > 0 && (uint32_t)cu >= tau;
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    int32_t at = -1;
+    uint32_t parts = in ? ((uint32_t)cu + kRadeChunk - 1) / kRadeChunk : 0u;
+    if (m) {
+      uint32_t base = 0, inc = parts;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+      uint32_t cbase = 0;
+      if (lane == 0) {
+        if (!all) base = atomicAdd(&ctl->count, (uint32_t)__popc(m));
+        cbase = atomicAdd(&ctl->nchunks, total);
+      }
+      base = __shfl_sync(0xffffffffu, base, 0);
+      cbase = __shfl_sync(0xffffffffu, cbase, 0);
+      if (in) {
+        at = all ? (int32_t)u : (int32_t)(base + __popc(m & ((1u << lane) - 1u)));
+        for (uint32_t q = 0; q < parts; ++q) chunks[cbase + inc - parts + q] = make_uint2((uint32_t)at, q);
+      }
+    }
+    if (u < n && !all) idx[u] = at;
+    if (all && u < n) at = (int32_t)u;
+    if (at >= 0) {
+      list[at] = (int32_t)u;
+      hc[at] = cu;
+    }
+  }
+}
+
+// Members as list entries (-1: not listed), so that a pick does not look them up.
+__global__ void __launch_bounds__(256) k_heavy_members(const int32_t *__restrict__ hmem, int64_t total,
+                                                       const int32_t *__restrict__ idx, int32_t *out) {
+  for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < total; e += (int64_t)gridDim.x * 256)
+    out[e] = idx[hmem[e]];
+}
+
+void heavy_list_all(const int32_t *c, int32_t n, HeavyCtl *ctl, int32_t *list, int32_t *hc, uint2 *chunks,
+                    cudaStream_t st) {
+  k_heavy_list<<<grid_for((size_t)n, 256 * 4, sm_count() * 4), 256, 0, st>>>(c, n, true, ctl, list, hc, nullptr, chunks);
+}
+
+// Chunks that the rows of `nodes` nodes can have.
+static size_t heavy_chunks_most(const cen_job *job, size_t nodes) {
+  return nodes + (size_t)job->members / kRadeChunk + 1;
+}
+
+// The heavy nodes of the current sample (incidence current), on the job's stream.
+void build_heavy(cen_job *job) {
+  if (job->heavy_m == job->m) return;
+  cudaStream_t st = job->st;
+  Stats *S = &job->stats;
+  const int32_t n = job->g->n;
+  const bool all = n <= kHeavyMax;
+  const size_t most = all ? (size_t)n : (size_t)kHeavyMax;
+  job->hctl.ensure(sizeof(HeavyCtl), st);
+  job->hlist.ensure(4 * most, st);
+  job->hc.ensure(4 * most, st);
+  job->hidx.ensure(all ? 4 : 4 * (size_t)n, st);
+  job->hchunks.ensure(8 * heavy_chunks_most(job, most), st);
+  HeavyCtl *ctl = job->hctl.as<HeavyCtl>();
+  CEN_CK(cudaMemsetAsync(ctl, 0, all ? offsetof(HeavyCtl, hist) : sizeof(HeavyCtl), st));
+  if (!all)
+    launch(S, K_TRANSPOSE, st, [&] {
+      k_heavy_hist<<<grid_for((size_t)n, 256 * 8, sm_count() * 4), 256, 0, st>>>(job->c.as<int32_t>(), n, ctl);
+    });
+  launch(S, K_TRANSPOSE, st, [&] {
+    k_heavy_list<<<grid_for((size_t)n, 256 * 4, sm_count() * 4), 256, 0, st>>>(
+        job->c.as<int32_t>(), n, all, ctl, job->hlist.as<int32_t>(), job->hc.as<int32_t>(), job->hidx.as<int32_t>(),
+        job->hchunks.as<uint2>());
+  });
+  if (!all && job->members) {
+    job->hmemh.ensure(4 * (size_t)job->members, st);
+    launch(S, K_TRANSPOSE, st, [&] {
+      k_heavy_members<<<grid_for((size_t)job->members, 256 * 4), 256, 0, st>>>(
+          job->hmem.as<int32_t>(), job->members, job->hidx.as<int32_t>(), job->hmemh.as<int32_t>());
+    });
+  }
+  job->heavy_m = job->m;
+}
+
+HeavyView heavy_view(const cen_job *job) {
+  return HeavyView{job->hctl.as<HeavyCtl>(), job->hlist.as<int32_t>(), job->hc.as<int32_t>(),
+                   job->hchunks.as<uint2>()};
+}
+
 // ---------------------------------------------------------------- greedy
 // Control words: key[2] (ping-pong argmax keys), covered count, picks, done.
 struct GreedyCtl {
@@ -62,7 +213,8 @@ struct GreedyCtl {
   unsigned long long covered;
   int size;
   int done;
-  int S[1];  // k entries follow
+  int short_;  // a pick among the heavy nodes fell below tau: all nodes are needed
+  int S[1];    // k entries follow
 };
 
 __global__ void k_gain_init(const int32_t *__restrict__ c, int32_t *gain, int32_t n) {
@@ -180,86 +332,142 @@ __global__ void __launch_bounds__(256) k_greedy_all(const int64_t *__restrict__ 
 
 // All k iterations in one thread-block cluster of C CTAs (16 where the device
 // allows clusters that large, else 8), the gains held in the CTAs' shared
-// memory (CTA r owns nodes [r per, (r+1) per)).
-// Per iteration: each CTA takes the largest key of its nodes (the same key as
-// k_greedy_all: largest gain, lowest id), a cluster barrier, every CTA reads
-// the others' keys through distributed shared memory and so picks the same
-// u*; then a thread per incident sample of u* sets the sample's covered bit
-// and, if it was not set, decrements the gains of the sample's members in
-// their owners' shared memory; another cluster barrier.  The picks and counts
-// are those of k_greedy_all.  A cluster is launched only when all of its CTAs
-// are resident at once, so the barriers always complete.
+// memory: item i (a heavy node's list entry, or with HEAVY = false node i) is
+// CTA i % C's.  Per iteration: each CTA takes the largest key of its items (the
+// same key as k_greedy_all: largest gain, lowest id), a cluster barrier, every
+// CTA reads the others' keys through distributed shared memory and so picks
+// the same u*; then a thread per incident sample of u* sets the sample's
+// covered bit and, if it was not set, decrements the gains of the sample's
+// members in their owners' shared memory; another cluster barrier.  The picks
+// and counts are those of k_greedy_all.  A cluster is launched only when all
+// of its CTAs are resident at once, so the barriers always complete.
+//
+// Over the heavy nodes a CTA holds at most 1,024 gains (two keys a thread), so
+// a pick costs its two barriers and the chain of loads of the picked row, some
+// 3.2 us: R-MAT 18, m = 65,536, k = 50: 0.21 -> 0.16 ms; directed R-MAT 22, k =
+// 100, whose 4.2 million gains no cluster holds: 3.2 -> 0.37 ms against the
+// grid form; the rewired grid of 4.2 million nodes, with samples of 36 members:
+// 4.0 -> 0.26 ms (1.7 with one lane a sample).
 constexpr int kGreedyClusterMax = 16;  // non-portable; 8 is the portable size
-// 512 threads: cheaper barriers per pick than 1,024 (measured 0.215 vs 0.23 ms per R-MAT 18
-// round with 16 CTAs; 0.24 vs 0.25 ms with 8)
+// 512 threads: cheaper barriers per pick than 1,024 (measured over all nodes 0.215 vs 0.23 ms per
+// R-MAT 18 round with 16 CTAs; 0.24 vs 0.25 ms with 8; over the heavy nodes 16 and 8 CTAs are equal)
 constexpr int kGreedyThreads = 512;
 
+template <bool HEAVY>
 __global__ void __launch_bounds__(kGreedyThreads, 1)
-    k_greedy_cluster(const int32_t *__restrict__ c, const int64_t *__restrict__ noff,
+    k_greedy_cluster(const int32_t *__restrict__ c, HeavyView H, const int64_t *__restrict__ noff,
                      const int32_t *__restrict__ nsamp, const int64_t *__restrict__ hoff,
-                     const int32_t *__restrict__ hmem, int32_t n, int32_t per, uint32_t *covered, GreedyCtl *ctl,
-                     int k) {
-  extern __shared__ int32_t s_gain[];
-  __shared__ unsigned long long s_wbest[kGreedyThreads / 32];
-  __shared__ unsigned long long s_best, s_key;
+                     const int32_t *__restrict__ hmem, int32_t n, uint32_t *covered, GreedyCtl *ctl, int k, int lg) {
+  extern __shared__ int64_t s_items[];
+  __shared__ uint32_t s_wgain[kGreedyThreads / 32], s_wid[kGreedyThreads / 32];
+  // the CTA's best and the cluster's: the node's complement (so that larger wins), its gain, its incidence row
+  struct __align__(16) Best {
+    uint32_t id, gain;
+    int32_t len, pad;
+    int64_t r0, pad2;
+  };
+  __shared__ Best s_best, s_pick;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int32_t u0 = rank * per, u1 = min(n, u0 + per);
-  for (int32_t u = u0 + tid; u < u1; u += kGreedyThreads) s_gain[u - u0] = c[u];
+  const int C = (int)cl.num_blocks(), lgC = 31 - __clz(C);
+  const int32_t items = HEAVY ? (int32_t)H.ctl->count : n;
+  const uint32_t tau = HEAVY ? (uint32_t)H.ctl->tau : 1u;
+  const int32_t mine = (items - rank + C - 1) >> lgC;  // items rank, rank + C, ...
+  const int32_t per = (items + C - 1) >> lgC;
+  int64_t *s_row = s_items;                                        // first incidence of an item (HEAVY)
+  int32_t *s_gain = (int32_t *)(s_items + (HEAVY ? per : 0));
+  int32_t *s_id = s_gain + per, *s_len = s_id + per;               // its node and c_u (HEAVY)
+  for (int32_t i = tid; i < mine; i += kGreedyThreads) {
+    if (HEAVY) {
+      const int32_t u = H.list[i * C + rank], cu = H.c[i * C + rank];
+      s_gain[i] = cu;
+      s_len[i] = cu;
+      s_id[i] = u;
+      s_row[i] = noff[u];
+    } else {
+      s_gain[i] = c[i * C + rank];
+    }
+  }
   cl.sync();
-  const int64_t gt = (int64_t)rank * kGreedyThreads + tid;
-  const int C = (int)cl.num_blocks();
-  const int64_t nthreads = (int64_t)C * kGreedyThreads;
+  // a sample's members are dealt to 2^lg lanes
+  const int gl = tid & ((1 << lg) - 1);
+  const unsigned gmask = (lg == 5 ? 0xffffffffu : (1u << (1 << lg)) - 1u) << (lane & ~((1 << lg) - 1));
+  const int64_t gt = ((int64_t)rank * kGreedyThreads + tid) >> lg;
+  const int64_t ngroups = ((int64_t)C * kGreedyThreads) >> lg;
   for (int it = 0; it < k; ++it) {
-    unsigned long long best = 0;
-    for (int32_t u = u0 + tid; u < u1; u += kGreedyThreads) {
-      const unsigned long long key = ((unsigned long long)(uint32_t)s_gain[u - u0] << 32) | (0xFFFFFFFFu - (uint32_t)u);
-      best = key > best ? key : best;
-    }
-    for (int o = 16; o; o >>= 1) {
-      const unsigned long long y = __shfl_xor_sync(0xffffffffu, best, o);
-      best = y > best ? y : best;
-    }
-    if (lane == 0) s_wbest[wid] = best;
-    __syncthreads();
-    if (wid == 0) {
-      best = lane < kGreedyThreads / 32 ? s_wbest[lane] : 0ull;
-      for (int o = 16; o; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, best, o);
-        best = y > best ? y : best;
+    uint32_t bg = 0, bi = 0;  // the thread's best gain, and the complement of its node
+    int32_t bat = 0;
+    for (int32_t i = tid; i < mine; i += kGreedyThreads) {
+      const uint32_t g = (uint32_t)s_gain[i], id = 0xFFFFFFFFu - (HEAVY ? (uint32_t)s_id[i] : (uint32_t)(i * C + rank));
+      if (g > bg || (g == bg && id > bi)) {
+        bg = g;
+        bi = id;
+        bat = i;
       }
-      if (lane == 0) s_best = best;
     }
-    cl.sync();  // every CTA's key is in place
-    if (wid == 0) {
-      unsigned long long key = lane < C ? *cl.map_shared_rank(&s_best, lane) : 0ull;
-      for (int o = 16; o; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, key, o);
-        key = y > key ? y : key;
-      }
-      if (lane == 0) s_key = key;
+    // the warp's best, then (every warp for itself) the CTA's
+    uint32_t g = __reduce_max_sync(0xffffffffu, bg);
+    uint32_t id = __reduce_max_sync(0xffffffffu, bg == g ? bi : 0u);
+    if (lane == 0) {
+      s_wgain[wid] = g;
+      s_wid[wid] = id;
     }
     __syncthreads();
-    const unsigned long long key = s_key;
-    const uint32_t g = (uint32_t)(key >> 32);
-    if (g == 0) break;  // every CTA holds the same key: all leave together
-    const int32_t u = (int32_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFu));
+    const uint32_t wg = lane < kGreedyThreads / 32 ? s_wgain[lane] : 0u;
+    const uint32_t wi = lane < kGreedyThreads / 32 ? s_wid[lane] : 0u;
+    g = __reduce_max_sync(0xffffffffu, wg);
+    id = __reduce_max_sync(0xffffffffu, wg == g ? wi : 0u);
+    if (g == 0) {
+      if (tid == 0) s_best.gain = 0;
+    } else if (bg == g && bi == id) {  // one thread holds it
+      const int64_t r = HEAVY ? s_row[bat] : noff[bat * C + rank];
+      s_best.gain = g;
+      s_best.id = id;
+      s_best.r0 = r;
+      s_best.len = HEAVY ? s_len[bat] : (int32_t)(noff[bat * C + rank + 1] - r);
+    }
+    cl.sync();  // every CTA's best is in place
+    if (wid == 0) {
+      uint4 o = make_uint4(0, 0, 0, 0);
+      int64_t r = 0;
+      if (lane < C) {
+        const Best *from = cl.map_shared_rank(&s_best, lane);
+        o = *(const uint4 *)from;
+        r = from->r0;
+      }
+      const uint32_t pg = __reduce_max_sync(0xffffffffu, o.y);
+      const uint32_t pi = __reduce_max_sync(0xffffffffu, o.y == pg ? o.x : 0u);
+      if (pg == 0 ? lane == 0 : o.y == pg && o.x == pi) {
+        s_pick.gain = pg;
+        s_pick.id = pi;
+        s_pick.len = (int32_t)o.z;
+        s_pick.r0 = r;
+      }
+    }
+    __syncthreads();
+    g = s_pick.gain;
+    if (g < tau) {  // nothing left to cover (tau = 1), or a lighter node may come next
+      if (HEAVY && tau > 1 && rank == 0 && tid == 0) ctl->short_ = 1;
+      break;  // every CTA holds the same pick: all leave together
+    }
+    const int64_t r0 = s_pick.r0, r1 = r0 + s_pick.len;
     if (rank == 0 && tid == 0) {
-      ctl->S[it] = u;
+      ctl->S[it] = (int32_t)(0xFFFFFFFFu - s_pick.id);
       ctl->size = it + 1;
       ctl->covered += g;
     }
-    const int64_t r0 = noff[u], r1 = noff[u + 1];
-    for (int64_t q = r0 + gt; q < r1; q += nthreads) {
+    for (int64_t q = r0 + gt; q < r1; q += ngroups) {
       const int32_t j = nsamp[q];
       const uint32_t mask = 1u << (j & 31);
       const int64_t e0 = hoff[j], e1 = hoff[j + 1];  // loaded alongside the covered bit
-      if (atomicOr(&covered[j >> 5], mask) & mask) continue;  // covered by an earlier pick
-      for (int64_t e = e0; e < e1; ++e) {
-        const int32_t w = hmem[e];
-        const int owner = w / per;
-        atomicSub(cl.map_shared_rank(s_gain + (w - owner * per), owner), 1);
+      uint32_t old = 0;
+      if (gl == 0) old = atomicOr(&covered[j >> 5], mask);
+      if (lg) old = __shfl_sync(gmask, old, 0, 1 << lg);
+      if (old & mask) continue;  // covered by an earlier pick
+      for (int64_t e = e0 + gl; e < e1; e += 1 << lg) {
+        const int32_t i = hmem[e];
+        if (!HEAVY || i >= 0) atomicSub(cl.map_shared_rank(s_gain + (i >> lgC), i & (C - 1)), 1);
       }
     }
     cl.sync();  // every gain update has landed before the next argmax
@@ -273,36 +481,79 @@ constexpr int64_t kGreedyClusterMaxPer = (227 * 1024 - 2048) / 4;
 
 size_t greedy_result_bytes(int32_t k) { return sizeof(GreedyCtl) + 4 * (size_t)k; }
 
-// Whether a cluster of C CTAs of k_greedy_cluster with `smem` bytes of gains
-// can be resident on this device (the kernel's shared-memory limit is raised,
-// and clusters over 8 allowed, once per process).
-static bool greedy_cluster_ready(int C, size_t smem) {
+// Whether a cluster of C CTAs of `kernel` with `smem` bytes can be resident on
+// this device (the kernel's shared-memory limit is raised, and clusters over 8
+// allowed, once per device).
+template <class K>
+static bool greedy_cluster_ready(K kernel, int C, size_t smem) {
   static std::mutex mu;
-  static int attr_ok = -1, big_ok = -1;
+  static std::map<std::pair<int, const void *>, int> attr;  // 1: set, 2: clusters over 8 too
+  int dev = 0;
+  CEN_CK(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(mu);
-  if (attr_ok < 0) {
-    attr_ok = cudaFuncSetAttribute(k_greedy_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(kGreedyClusterMaxPer * 4)) == cudaSuccess;
+  int &have = attr[{dev, (const void *)kernel}];
+  if (!have) {
+    have = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(kGreedyClusterMaxPer * 4 + 8)) == cudaSuccess ? 1 : -1;
     cudaGetLastError();
-    big_ok = cudaFuncSetAttribute(k_greedy_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    if (have > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+      have = 2;
     cudaGetLastError();
   }
-  if (!attr_ok || (C > 8 && !big_ok)) return false;
+  if (have < 0 || (C > 8 && have < 2)) return false;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(C);
   cfg.blockDim = dim3(kGreedyThreads);
   cfg.dynamicSmemBytes = smem;
-  cfg.attrs = attr;
+  cfg.attrs = at;
   cfg.numAttrs = 1;
   int clusters = 0;
-  const bool ok = cudaOccupancyMaxActiveClusters(&clusters, k_greedy_cluster, &cfg) == cudaSuccess && clusters >= 1;
+  const bool ok = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1;
   cudaGetLastError();
   return ok;
+}
+
+// Enqueues k_greedy_cluster<HEAVY> over `items` gains in the largest cluster
+// that holds them; false when none does.  Diagnostic: CEN_GREEDY_CLUSTER=8
+// keeps the portable cluster size.
+template <bool HEAVY>
+static bool greedy_cluster(cen_job *job, int32_t k, int64_t items, cudaStream_t run, GreedyCtl *ctl) {
+  const char *size_env = getenv("CEN_GREEDY_CLUSTER");
+  // the members of a sample as list entries, and lanes for about its mean number of members
+  const int32_t *members = (HEAVY && job->g->n > kHeavyMax ? job->hmemh : job->hmem).as<int32_t>();
+  int lg = 0;
+  while (lg < 5 && (double)((int64_t)2 << lg) * (double)job->m <= (double)job->members) ++lg;
+  for (int C : {kGreedyClusterMax, 8}) {
+    if (C > 8 && size_env && atoi(size_env) == 8) continue;
+    const int64_t per = (items + C - 1) / C;
+    const size_t smem = (size_t)per * (HEAVY ? 20 : 4) + 8;
+    if (smem > (size_t)kGreedyClusterMaxPer * 4 + 8 || !greedy_cluster_ready(k_greedy_cluster<HEAVY>, C, smem)) continue;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(kGreedyThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = run;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    launch(&job->stats, K_GREEDY, run, [&] {
+      CEN_CK(cudaLaunchKernelEx(&cfg, k_greedy_cluster<HEAVY>, (const int32_t *)job->c.as<int32_t>(), heavy_view(job),
+                                (const int64_t *)job->noff.as<int64_t>(), (const int32_t *)job->nsamp.as<int32_t>(),
+                                (const int64_t *)job->hoff.as<int64_t>(), members, job->g->n,
+                                job->covered.as<uint32_t>(), ctl, (int)k, lg));
+    });
+    return true;
+  }
+  return false;
 }
 
 // Sizes the greedy workspace for k picks (allocations ordered on the job's
@@ -315,46 +566,22 @@ void greedy_prepare(cen_job *job, int32_t k) {
   job->gctl.ensure(greedy_result_bytes(k), st);
 }
 
-// Enqueues greedyCover(k) on stream `run` (after greedy_prepare); the result
-// reaches hdst (pinned, greedy_result_bytes(k)) once `run` has drained.
-void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst) {
+// Enqueues greedyCover(k) on stream `run` (after greedy_prepare), over the
+// heavy nodes or over all; the result reaches hdst (pinned,
+// greedy_result_bytes(k)) once `run` has drained.
+void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool heavy) {
   Stats *St = &job->stats;
   const int32_t n = job->g->n;
   const size_t cbytes = greedy_result_bytes(k);
   CEN_CK(cudaMemsetAsync(job->covered.p, 0, 4 * ((job->m + 31) / 32 + 1), run));
   CEN_CK(cudaMemsetAsync(job->gctl.p, 0, cbytes, run));
   GreedyCtl *ctl = job->gctl.as<GreedyCtl>();
-  // diagnostics: CEN_GREEDY_GRID=1 keeps the cooperative grid form, CEN_GREEDY_CLUSTER=8 the
-  // portable cluster size
+  // diagnostic: CEN_GREEDY_GRID=1 keeps the cooperative grid form
   const char *grid_env = getenv("CEN_GREEDY_GRID");
-  const char *size_env = getenv("CEN_GREEDY_CLUSTER");
   const bool grid_form = grid_env && grid_env[0] == '1';
-  int C = 0;
-  for (int c : {kGreedyClusterMax, 8}) {
-    if (grid_form || C || (c > 8 && size_env && atoi(size_env) == 8)) continue;
-    const int64_t per_c = ((int64_t)n + c - 1) / c;
-    if (per_c <= kGreedyClusterMaxPer && greedy_cluster_ready(c, (size_t)per_c * 4)) C = c;
-  }
-  if (C) {
-    const int64_t per = ((int64_t)n + C - 1) / C;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(kGreedyThreads);
-    cfg.dynamicSmemBytes = (size_t)per * 4;
-    cfg.stream = run;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    launch(St, K_GREEDY, run, [&] {
-      CEN_CK(cudaLaunchKernelEx(&cfg, k_greedy_cluster, (const int32_t *)job->c.as<int32_t>(),
-                                (const int64_t *)job->noff.as<int64_t>(), (const int32_t *)job->nsamp.as<int32_t>(),
-                                (const int64_t *)job->hoff.as<int64_t>(), (const int32_t *)job->hmem.as<int32_t>(), n,
-                                (int32_t)per, job->covered.as<uint32_t>(), ctl, (int)k));
-    });
+  const bool done = !grid_form && (heavy ? greedy_cluster<true>(job, k, std::min<int64_t>(n, kHeavyMax), run, ctl)
+                                         : greedy_cluster<false>(job, k, n, run, ctl));
+  if (done) {
     CEN_CK(cudaMemcpyAsync(hdst, ctl, cbytes, cudaMemcpyDeviceToHost, run));
     return;
   }
@@ -391,12 +618,23 @@ void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst) {
   CEN_CK(cudaMemcpyAsync(hdst, ctl, cbytes, cudaMemcpyDeviceToHost, run));
 }
 
-// S, |S| and the covered count from the copied result.
-void greedy_result(const void *h, int32_t *S, int32_t *S_size, uint64_t *covered) {
+// S, |S| and the covered count from the copied result; false when the heavy
+// nodes did not decide every pick.
+bool greedy_result(const void *h, int32_t *S, int32_t *S_size, uint64_t *covered) {
   const GreedyCtl *hc = (const GreedyCtl *)h;
+  if (hc->short_) return false;
   *S_size = hc->size;
   *covered = hc->covered;
   for (int i = 0; i < hc->size; ++i) S[i] = hc->S[i];
+  return true;
+}
+
+// greedyCover over all nodes, on the job's stream (greedy_prepare done).
+void greedy_over_all(cen_job *job, int32_t k, void *h, int32_t *S, int32_t *S_size, uint64_t *covered) {
+  job->greedy_all = true;  // the job's later samples spread over as many nodes
+  greedy_enqueue(job, k, job->st, h, false);
+  CEN_CK(cudaStreamSynchronize(job->st));
+  greedy_result(h, S, S_size, covered);
 }
 
 // ------------------------------------------- greedyCover one pick at a time
@@ -492,11 +730,12 @@ void greedy_cover(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint64_t
   CEN_REQUIRE(k >= 1, CEN_EINVAL, "cen_greedy_cover: k must be >= 1");
   Range range("cen_greedy_cover");
   build_incidence(job);
+  build_heavy(job);
   greedy_prepare(job, k);
   void *h = host_staging(job, greedy_result_bytes(k));
-  greedy_enqueue(job, k, job->st, h);
+  greedy_enqueue(job, k, job->st, h, !job->greedy_all);
   CEN_CK(cudaStreamSynchronize(job->st));
-  greedy_result(h, S, S_size, covered);
+  if (!greedy_result(h, S, S_size, covered)) greedy_over_all(job, k, h, S, S_size, covered);
 }
 
 }  // namespace cen

@@ -132,10 +132,16 @@ struct cen_job {
   // node -> sample incidence (rebuilt lazily when m changed)
   cen::DevBuf c, noff, nsamp, cursor;
   uint64_t inc_m = ~0ull;
+  // heavy nodes of the sample (heavy.cuh) and whether the last greedy / AMCERA needed all nodes
+  cen::DevBuf hctl, hlist, hc, hidx, hchunks, hmemh;
+  uint64_t heavy_m = ~0ull;
+  bool greedy_all = false, rade_all = false;
   // greedy workspace
   cen::DevBuf gain, covered, gctl;
   // AMCERA workspace
   cen::DevBuf R, selh, selst;
+  cen::DevBuf Rh, hchunks_all, hctl_all, hlist_all, hc_all;  // over the heavy nodes; the chunks of all rows
+  uint64_t rade_all_m = ~0ull;      // sample size that R holds every node's row of
   int32_t rade_valid_k = -1;
   // greedyCover and AMCERA side by side (cen_cover_and_mcera)
   cen::AuxStream aux;
@@ -200,12 +206,15 @@ void shard_rade(cen_job *job, int32_t *R_out, int32_t *b);
 void shard_topk(cen_job *job, const int32_t *vals, int32_t nrows, int32_t k, int64_t *out);
 size_t greedy_result_bytes(int32_t k);
 void greedy_prepare(cen_job *job, int32_t k);
-void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst);
-void greedy_result(const void *h, int32_t *S, int32_t *S_size, uint64_t *covered);
+void build_heavy(cen_job *job);
+void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool heavy);
+bool greedy_result(const void *h, int32_t *S, int32_t *S_size, uint64_t *covered);
+void greedy_over_all(cen_job *job, int32_t k, void *h, int32_t *S, int32_t *S_size, uint64_t *covered);
+void rade_for_copy(cen_job *job);
 size_t mcera_result_bytes(const cen_job *job);
 void mcera_prepare(cen_job *job, int32_t k);
-void mcera_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst);
-void mcera_result(cen_job *job, int32_t k, const void *h, int64_t *Rnum, int64_t *Wnum, int32_t *b);
+void mcera_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool heavy);
+bool mcera_result(cen_job *job, int32_t k, const void *h, int64_t *Rnum, int64_t *Wnum, int32_t *b);
 void cover_and_mcera(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint64_t *covered, int64_t *Rnum,
                      int64_t *Wnum, int32_t *b);
 void graph_build(cen_graph *g, const int64_t *off, const int32_t *col, bool on_device, Stats *S);
