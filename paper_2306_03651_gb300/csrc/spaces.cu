@@ -20,185 +20,226 @@ namespace cen {
 
 namespace {
 
-constexpr int kWalkWarps = 8;      // warps (samples) per block of the walk kernel
+constexpr int kWalkThreads = 128;  // block of the walk kernel
 constexpr int kMaxKappa = 1024;
 
-// Warp per sample.  The walk (at most kappa nodes after s) sits in shared
-// memory; each step counts the current node's out-neighbours that are not on
-// it, 32 arcs at a time, and takes the r-th of them.
-__global__ void __launch_bounds__(32 * kWalkWarps) k_kpath(uint64_t j0, uint64_t count, int32_t n, int kappa,
-                                                           const int64_t *__restrict__ off,
-                                                           const int32_t *__restrict__ col, SampleKey key,
-                                                           int32_t *ps, int32_t *pt, int32_t *pd, int32_t *out,
-                                                           const int64_t *__restrict__ hoff, int *bmax,
-                                                           unsigned long long *units) {
+// First position in the sorted c[lo, hi) whose value is >= w.
+__device__ __forceinline__ int64_t lower_bound32(const int32_t *__restrict__ c, int64_t lo, int64_t hi, int32_t w) {
+  while (lo < hi) {
+    const int64_t mid = lo + ((hi - lo) >> 1);
+    if (c[mid] < w)
+      lo = mid + 1;
+    else
+      hi = mid;
+  }
+  return lo;
+}
+
+// GS lanes per sample.  The walk (at most kappa nodes after s) sits in shared
+// memory.  At a step the lanes look the walk's nodes up in the current node's
+// sorted row: the row less those found are the free out-neighbours, and the
+// r-th of them is the least position i with i = r + (found positions <= i),
+// reached from i = r by repetition.  So a step costs a binary search per walk
+// node, side by side, where counting and finding the free arcs one by one
+// reads a hub's row of thousands twice (R-MAT 18, kappa = 8, 65,536 walks:
+// 2.0 -> 0.10 ms).  Bound by the latency of a step's chain of loads; 8 lanes
+// hold all nodes of a walk of kappa <= 8, so four walks share a warp.
+template <int GS>
+__global__ void __launch_bounds__(kWalkThreads) k_kpath(uint64_t j0, uint64_t count, int32_t n, int kappa,
+                                                        const int64_t *__restrict__ off,
+                                                        const int32_t *__restrict__ col, SampleKey key, int32_t *ps,
+                                                        int32_t *pt, int32_t *pd, int32_t *out,
+                                                        const int64_t *__restrict__ hoff, int *bmax,
+                                                        unsigned long long *units) {
   extern __shared__ int32_t walk_sh[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  int32_t *walk = walk_sh + (size_t)wib * kappa;
-  const uint64_t nw = (uint64_t)gridDim.x * kWalkWarps;
-  unsigned long long arcs = 0;
+  constexpr int kGroups = kWalkThreads / GS;
+  const int gl = threadIdx.x & (GS - 1), gib = threadIdx.x / GS, lane = threadIdx.x & 31;
+  const unsigned gmask = GS == 32 ? 0xffffffffu : ((1u << GS) - 1u) << (lane & ~(GS - 1));
+  int32_t *walk = walk_sh + (size_t)gib * 2 * kappa;  // then the found positions
+  int32_t *found = walk + kappa;
+  const uint64_t ng = (uint64_t)gridDim.x * kGroups;
+  unsigned long long probes = 0;
   int mymax = 0;
-  for (uint64_t i = (uint64_t)blockIdx.x * kWalkWarps + wib; i < count; i += nw) {
+  for (uint64_t i = (uint64_t)blockIdx.x * kGroups + gib; i < count; i += ng) {
     const uint64_t j = j0 + i;
-    const int32_t s = (int32_t)uniform_below64(key.seed, key.id(j), kPurposeS, (uint64_t)n);
-    const int32_t l = 1 + (int32_t)uniform_below64(key.seed, key.id(j), kPurposeT, (uint64_t)kappa);
+    int32_t draw = 0;  // lane 0 draws s, lane 1 the length
+    if (gl < 2)
+      draw = (int32_t)uniform_below64(key.seed, key.id(j), gl ? kPurposeT : kPurposeS, (uint64_t)(gl ? kappa : n));
+    const int32_t s = __shfl_sync(gmask, draw, 0, GS);
+    const int32_t l = 1 + __shfl_sync(gmask, draw, 1, GS);
     int32_t cur = s, len = 0;
     for (int32_t step = 0; step < l; ++step) {
-      const int64_t e0 = off[cur], e1 = off[cur + 1];
-      // free out-neighbours: not s and not on the walk
-      unsigned long long nfree = 0;
-      for (int64_t b = e0; b < e1; b += 32) {
-        const int64_t e = b + lane;
-        bool fr = false;
-        if (e < e1) {
-          const int32_t w = col[e];
-          fr = w != s;
-          for (int q = 0; q < len && fr; ++q) fr = walk[q] != w;
+      const int64_t e0 = off[cur];
+      const int32_t deg = (int32_t)(off[cur + 1] - e0);
+      const int32_t *__restrict__ row = col + e0;
+      int32_t nfound = 0;  // of s and the walk's nodes, in the row
+      for (int q = gl; q - gl <= len; q += GS) {
+        int32_t at = -1;
+        if (q <= len) {
+          const int32_t w = q ? walk[q - 1] : s;
+          const int32_t p = (int32_t)lower_bound32(row, 0, deg, w);
+          if (p < deg && row[p] == w) at = p;
         }
-        nfree += __popc(__ballot_sync(0xffffffffu, fr));
+        const unsigned m = __ballot_sync(gmask, at >= 0);
+        if (at >= 0) found[nfound + __popc(m & ((1u << lane) - 1u))] = at;
+        nfound += __popc(m);
       }
-      arcs += (unsigned long long)(e1 - e0);
-      if (nfree == 0) break;
-      unsigned long long r = uniform_below64(key.seed, key.id(j), kPurposeWalk0 + (uint32_t)step, nfree);
-      int32_t next = -1;
-      for (int64_t b = e0; b < e1 && next < 0; b += 32) {
-        const int64_t e = b + lane;
-        bool fr = false;
-        int32_t w = -1;
-        if (e < e1) {
-          w = col[e];
-          fr = w != s;
-          for (int q = 0; q < len && fr; ++q) fr = walk[q] != w;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, fr);
-        const unsigned c = (unsigned)__popc(m);
-        if (r < c) {  // the r-th free arc of this chunk
-          unsigned mm = m;
-          for (unsigned q = 0; q < (unsigned)r; ++q) mm &= mm - 1;
-          next = __shfl_sync(0xffffffffu, w, __ffs(mm) - 1);
-        } else {
-          r -= c;
-        }
+      probes += (unsigned long long)(len + 1);
+      if (nfound == deg) break;
+      const int32_t r =
+          (int32_t)uniform_below64(key.seed, key.id(j), kPurposeWalk0 + (uint32_t)step, (uint64_t)(deg - nfound));
+      __syncwarp(gmask);
+      int32_t at = r;
+      for (;;) {
+        int32_t below = 0;
+        for (int q = gl; q - gl < nfound; q += GS)
+          below += __popc(__ballot_sync(gmask, q < nfound && found[q] <= at));
+        if (r + below == at) break;
+        at = r + below;
       }
-      __syncwarp();
-      if (lane == 0) walk[len] = next;
-      __syncwarp();
+      cur = row[at];
+      if (gl == 0) walk[len] = cur;
+      __syncwarp(gmask);
       ++len;
-      cur = next;
     }
     if (out) {  // members at stride kappa, or at their place in the store when hoff is given
       int32_t *dst = hoff ? out + hoff[j] : out + (size_t)i * kappa;
-      for (int q = lane; q < len; q += 32) dst[q] = walk[q];
+      for (int q = gl; q < len; q += GS) dst[q] = walk[q];
     }
-    if (lane == 0) {
+    if (gl == 0) {
       ps[j] = s;
       pt[j] = l;
       pd[j] = len;
     }
     mymax = max(mymax, len);
-    __syncwarp();
+    __syncwarp(gmask);
   }
+  mymax = __reduce_max_sync(0xffffffffu, mymax);
+  probes = warp_sum(gl == 0 ? probes : 0ull);
   if (lane == 0) {
     if (mymax) atomicMax(bmax, mymax);
-    if (arcs) atomicAdd(units, arcs * 4ull);
+    if (probes) atomicAdd(units, probes * 4ull);
   }
 }
 
+// The largest i in [0, count) with a[i] <= x (a ascending, a[0] <= x), by a
+// whole warp: 32 probes a round.
+__device__ __forceinline__ int64_t warp_upper(const int64_t *__restrict__ a, int64_t count, int64_t x) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = 0, hi = count;  // a[lo] <= x, and a[hi] > x or hi = count
+  while (hi - lo > 1) {
+    const int64_t step = (hi - lo + 32) / 33;
+    const int64_t at = lo + (int64_t)(lane + 1) * step;
+    const bool le = at < hi && a[at] <= x;
+    const int c = __popc(__ballot_sync(0xffffffffu, le));  // the probes ascend
+    const int64_t nhi = lo + (int64_t)(c + 1) * step;
+    lo += (int64_t)c * step;
+    hi = nhi < hi ? nhi : hi;
+  }
+  return lo;
+}
+
 // Common neighbours w > v of u and v, ascending: the shorter row's entries
-// above v are looked up in the longer row by binary search (both rows are
-// sorted, so either order of the two rows gives the same ascending w).
-// Returns how many there are; with want >= 0, stops at the one of that rank
-// and returns it in *w_out.
-__device__ int64_t common_above(const int64_t *__restrict__ off, const int32_t *__restrict__ col, int32_t u, int32_t v,
-                                int64_t want, int32_t *w_out) {
-  int64_t a0 = off[u], a1 = off[u + 1], b0 = off[v], b1 = off[v + 1];
-  if (a1 - a0 > b1 - b0) {
-    const int64_t t0 = a0, t1 = a1;
-    a0 = b0;
-    a1 = b1;
-    b0 = t0;
-    b1 = t1;
+// above v, 128 at a time, are looked up in the longer row by binary search
+// (both rows are sorted, so either order of the two rows gives the same
+// ascending w).  A lane's four searches go side by side, so that their loads
+// overlap.  Returns how many there are; with want >= 0, stops at the one of
+// that rank and returns it in *w_out.  Called by a whole warp.
+__device__ __forceinline__ int32_t common_above(const int64_t *__restrict__ off, const int32_t *__restrict__ col,
+                                                int32_t u, int32_t v, int64_t want, int32_t *w_out) {
+  constexpr int U = 4;
+  const int lane = threadIdx.x & 31;
+  const int64_t u0 = off[u], v0 = off[v];
+  int32_t na = (int32_t)(off[u + 1] - u0), nb = (int32_t)(off[v + 1] - v0);
+  const int32_t *__restrict__ A = col + u0, *__restrict__ B = col + v0;
+  if (na > nb) {
+    const int32_t *t = A;
+    A = B;
+    B = t;
+    const int32_t nt = na;
+    na = nb;
+    nb = nt;
   }
-  {  // first entry of the shorter row above v
-    int64_t lo = a0, hi = a1;
-    while (lo < hi) {
-      const int64_t mid = lo + ((hi - lo) >> 1);
-      if (col[mid] <= v)
-        lo = mid + 1;
-      else
-        hi = mid;
+  int32_t c = 0;
+  for (int32_t a = (int32_t)lower_bound32(A, 0, na, v + 1); a < na && nb > 0; a += 32 * U) {
+    int32_t w[U], p[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      w[i] = a + 32 * i + lane < na ? A[a + 32 * i + lane] : 0x7fffffff;
+      p[i] = 0;
     }
-    a0 = lo;
-  }
-  int64_t c = 0;
-  for (int64_t a = a0; a < a1; ++a) {
-    const int32_t w = col[a];
-    int64_t lo = b0, hi = b1;
-    while (lo < hi) {
-      const int64_t mid = lo + ((hi - lo) >> 1);
-      if (col[mid] < w)
-        lo = mid + 1;
-      else
-        hi = mid;
+    int32_t len = nb;
+    while (len > 1) {
+      const int32_t half = len >> 1;
+#pragma unroll
+      for (int i = 0; i < U; ++i)
+        if (B[p[i] + half - 1] < w[i]) p[i] += half;
+      len -= half;
     }
-    b0 = lo;  // w ascends, so the search range only shrinks
-    if (lo < b1 && col[lo] == w) {
-      if (c == want) {
-        *w_out = w;
-        return c;
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+      const int32_t x = B[p[i]];  // the first entry >= w, or the last
+      unsigned m = __ballot_sync(0xffffffffu, x == w[i] && a + 32 * i + lane < na);
+      const int found = __popc(m);
+      if (want >= 0 && want < c + found) {
+        for (int64_t q = c; q < want; ++q) m &= m - 1;
+        *w_out = __shfl_sync(0xffffffffu, w[i], __ffs(m) - 1);
+        return (int32_t)want;
       }
-      ++c;
+      c += found;
     }
   }
   return c;
 }
 
-// Thread per arc: its triangle count (0 unless col > row).
-__global__ void k_tri_count(int32_t n, const int64_t *__restrict__ off, const int32_t *__restrict__ col,
-                            int64_t *cnt) {
-  for (int32_t u = blockIdx.x * blockDim.y + threadIdx.y; u < n; u += gridDim.x * blockDim.y)
-    for (int64_t e = off[u] + threadIdx.x; e < off[u + 1]; e += blockDim.x) {
+// Warp per run of kTriRun arcs: each arc's triangle count (0 unless col > row).
+// The lanes share an arc's row entries, so a hub's arcs do not run on in one
+// thread (R-MAT 16, the first job on a graph: 104 -> 1.2 ms).
+constexpr int kTriRun = 8;
+__global__ void __launch_bounds__(256) k_tri_count(int32_t n, int64_t nnz, const int64_t *__restrict__ off,
+                                                   const int32_t *__restrict__ col, int64_t *cnt) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nwarps = (int64_t)gridDim.x * 8;
+  for (int64_t b = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * kTriRun; b < nnz; b += nwarps * kTriRun) {
+    const int64_t end = b + kTriRun < nnz ? b + kTriRun : nnz;
+    int64_t u = warp_upper(off, (int64_t)n + 1, b);
+    int64_t mine = 0;
+    for (int64_t e = b; e < end; ++e) {
+      if (off[u + 1] <= e) u += warp_upper(off + u, (int64_t)n + 1 - u, e);
       const int32_t v = col[e];
-      cnt[e] = v > u ? common_above(off, col, u, v, -1, nullptr) : 0;
+      if (v <= u) continue;
+      const int64_t c = common_above(off, col, (int32_t)u, v, -1, nullptr);
+      if (e - b == lane) mine = c;
     }
+    if (lane < kTriRun && b + lane < end) cnt[b + lane] = mine;
+  }
 }
 
-// Thread per sample: rank r -> arc e (the last with tri_off[e] <= r) -> (u, v)
-// -> the common neighbour of rank r - tri_off[e].
-__global__ void k_tri_sample(uint64_t j0, uint64_t count, int32_t n, int64_t nnz, const int64_t *__restrict__ off,
-                             const int32_t *__restrict__ col, const int64_t *__restrict__ tri_off, SampleKey key,
-                             int32_t *ps, int32_t *pt, int32_t *pd, const int64_t *__restrict__ hoff, int32_t *hmem) {
+// Warp per sample: rank r -> arc e (the last with tri_off[e] <= r) -> (u, v)
+// -> the common neighbour of rank r - tri_off[e].  Bound by the latency of its
+// searches, 33-way for the arc and its row, and a binary search per lane among
+// the common neighbours.  R-MAT 16, 65,536 samples: 4.0 ms with a thread per
+// sample -> 0.21 ms
+__global__ void __launch_bounds__(256) k_tri_sample(uint64_t j0, uint64_t count, int32_t n, int64_t nnz,
+                                                    const int64_t *__restrict__ off, const int32_t *__restrict__ col,
+                                                    const int64_t *__restrict__ tri_off, SampleKey key, int32_t *ps,
+                                                    int32_t *pt, int32_t *pd, const int64_t *__restrict__ hoff,
+                                                    int32_t *hmem) {
+  const int lane = threadIdx.x & 31;
   const uint64_t T = (uint64_t)tri_off[nnz];
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (uint64_t)gridDim.x * blockDim.x) {
+  const uint64_t nwarps = (uint64_t)gridDim.x * 8;
+  for (uint64_t i = (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5); i < count; i += nwarps) {
     const uint64_t j = j0 + i;
     const int64_t r = (int64_t)uniform_below64(key.seed, key.id(j), kPurposeS, T);
-    int64_t lo = 0, hi = nnz + 1;  // upper bound of r in tri_off[0 .. nnz], minus one
-    while (lo < hi) {
-      const int64_t mid = lo + ((hi - lo) >> 1);
-      if (tri_off[mid] <= r)
-        lo = mid + 1;
-      else
-        hi = mid;
-    }
-    const int64_t e = lo - 1;
-    int32_t a = 0, b = n;  // the row holding arc e
-    while (b - a > 1) {
-      const int32_t mid = a + ((b - a) >> 1);
-      if (off[mid] <= e)
-        a = mid;
-      else
-        b = mid;
-    }
-    const int32_t u = a, v = col[e];
+    const int64_t e = warp_upper(tri_off, nnz + 1, r);
+    const int32_t u = (int32_t)warp_upper(off, (int64_t)n + 1, e), v = col[e];
     int32_t w = -1;
     common_above(off, col, u, v, r - tri_off[e], &w);
-    ps[j] = u;
-    pt[j] = v;
-    pd[j] = w;
-    const int64_t h = hoff[j];
-    hmem[h] = u;
-    hmem[h + 1] = v;
-    hmem[h + 2] = w;
+    if (lane < 3) {
+      const int32_t x = lane == 0 ? u : lane == 1 ? v : w;
+      (lane == 0 ? ps : lane == 1 ? pt : pd)[j] = x;
+      hmem[hoff[j] + lane] = x;
+    }
   }
 }
 
@@ -209,13 +250,20 @@ __global__ void k_tri_sample(uint64_t j0, uint64_t count, int32_t n, int64_t nnz
 void kpath_sample(cen_job *job, uint64_t j0, uint64_t count, int32_t *out, const int64_t *hoff) {
   const cen_graph *g = job->g;
   cudaStream_t st = job->st;
-  const size_t smem = sizeof(int32_t) * (size_t)job->kappa * kWalkWarps;
-  launch(&job->stats, K_SPACE, st, [&] {
-    k_kpath<<<grid_for(count, kWalkWarps, sm_count() * 16), 32 * kWalkWarps, smem, st>>>(
-        j0, count, g->n, job->kappa, g->off.as<int64_t>(), g->col.as<int32_t>(), job->key(), job->ps.as<int32_t>(),
-        job->pt.as<int32_t>(), job->pd.as<int32_t>(), out, hoff, job->bmax.as<int>(),
-        (unsigned long long *)(job->stats.d_units + K_SPACE));
-  });
+  auto go = [&](auto kernel, int gs) {
+    const int groups = kWalkThreads / gs;
+    const size_t smem = 2 * sizeof(int32_t) * (size_t)job->kappa * groups;
+    launch(&job->stats, K_SPACE, st, [&] {
+      kernel<<<grid_for(count, groups, sm_count() * 16), kWalkThreads, smem, st>>>(
+          j0, count, g->n, job->kappa, g->off.as<int64_t>(), g->col.as<int32_t>(), job->key(), job->ps.as<int32_t>(),
+          job->pt.as<int32_t>(), job->pd.as<int32_t>(), out, hoff, job->bmax.as<int>(),
+          (unsigned long long *)(job->stats.d_units + K_SPACE));
+    });
+  };
+  if (job->kappa <= 8)
+    go(k_kpath<8>, 8);
+  else
+    go(k_kpath<32>, 32);
 }
 
 // Triangle ranks of the graph (kept on the graph), and their total.
@@ -228,8 +276,8 @@ int64_t triangle_index(cen_job *job) {
     cnt.ensure(8 * (size_t)(g->nnz + 1), st);
     g->tri_off.ensure(8 * (size_t)(g->nnz + 1), st);
     launch(&job->stats, K_SPACE, st, [&] {
-      k_tri_count<<<grid_for((size_t)g->n, 8, sm_count() * 64), dim3(32, 8), 0, st>>>(g->n, g->off.as<int64_t>(),
-                                                                              g->col.as<int32_t>(), cnt.as<int64_t>());
+      k_tri_count<<<grid_for((size_t)g->nnz, 8 * kTriRun, sm_count() * 64), 256, 0, st>>>(
+          g->n, g->nnz, g->off.as<int64_t>(), g->col.as<int32_t>(), cnt.as<int64_t>());
     });
     exclusive_scan_i64(cnt.as<int64_t>(), g->tri_off.as<int64_t>(), (size_t)g->nnz, g->tri_off.as<int64_t>() + g->nnz,
                        job->scan_tmp, st, &job->stats);
@@ -248,7 +296,7 @@ void triangle_sample(cen_job *job, uint64_t j0, uint64_t count) {
   const cen_graph *g = job->g;
   cudaStream_t st = job->st;
   launch(&job->stats, K_SPACE, st, [&] {
-    k_tri_sample<<<grid_for(count, 256), 256, 0, st>>>(j0, count, g->n, g->nnz, g->off.as<int64_t>(),
+    k_tri_sample<<<grid_for(count, 8), 256, 0, st>>>(j0, count, g->n, g->nnz, g->off.as<int64_t>(),
                                                          g->col.as<int32_t>(), g->tri_off.as<int64_t>(), job->key(),
                                                          job->ps.as<int32_t>(), job->pt.as<int32_t>(),
                                                          job->pd.as<int32_t>(), job->hoff.as<int64_t>(),
