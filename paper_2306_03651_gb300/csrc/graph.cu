@@ -54,15 +54,70 @@ __global__ void k_check_loops(const int64_t *__restrict__ off, const int32_t *__
   }
 }
 
-// Arc list in CSR order: key = head, value = tail.
-__global__ void k_arcs_by_tail(const int64_t *off, const int32_t *col, int32_t n, uint32_t *key, uint32_t *val) {
+// The row that holds arc e of the offsets off[n + 1] (the last that starts at
+// or before it), by a whole warp: 32 probes a round.
+__device__ __forceinline__ int32_t warp_row(const int64_t *__restrict__ off, int32_t n, int64_t e) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = 0, hi = (int64_t)n + 1;
+  while (hi - lo > 1) {
+    const int64_t step = (hi - lo + 32) / 33, at = lo + (int64_t)(lane + 1) * step;
+    const int c = __popc(__ballot_sync(0xffffffffu, at < hi && off[at] <= e));
+    const int64_t nhi = lo + (int64_t)(c + 1) * step;
+    lo += (int64_t)c * step;
+    hi = nhi < hi ? nhi : hi;
+  }
+  return (int32_t)lo;
+}
+
+// Calls f(e, u) for every arc e with its row u.  A warp takes kArcRun
+// consecutive arcs, finds the rows of the first and the last, and each lane
+// searches its arcs' rows between them, so that work follows arcs and not
+// rows (a warp per row took 0.87 ms for 15.6 million R-MAT arcs, waiting on
+// the hubs' rows; this takes 0.10).
+constexpr int kArcRun = 256;
+template <class F>
+__device__ __forceinline__ void for_arcs(const int64_t *__restrict__ off, int32_t n, int64_t nnz, F &&f) {
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += nwarps) {
-    for (int64_t i = off[v] + lane; i < off[v + 1]; i += 32) {
-      key[i] = (uint32_t)col[i];
-      val[i] = (uint32_t)v;
+  for (int64_t b = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kArcRun; b < nnz; b += nwarps * kArcRun) {
+    const int64_t end = b + kArcRun < nnz ? b + kArcRun : nnz;
+    int32_t lo = warp_row(off, n, b);
+    const int32_t last = warp_row(off, n, end - 1);
+    for (int64_t e = b + lane; e < end; e += 32) {
+      int32_t hi = last;  // off[lo] <= e
+      while (lo < hi) {
+        const int32_t mid = lo + ((hi - lo + 1) >> 1);
+        if (off[mid] <= e)
+          lo = mid;
+        else
+          hi = mid - 1;
+      }
+      f(e, lo);
     }
+  }
+}
+
+// Arc list in CSR order: key = head, value = tail.
+__global__ void __launch_bounds__(256) k_arcs_by_tail(const int64_t *__restrict__ off, const int32_t *__restrict__ col,
+                                                      int32_t n, int64_t nnz, uint32_t *key, uint32_t *val) {
+  for_arcs(off, n, nnz, [&](int64_t e, int32_t u) {
+    key[e] = (uint32_t)col[e];
+    val[e] = (uint32_t)u;
+  });
+}
+
+// Sets roff[w] = at for the rows w in (lo, hi]: a lane's own when they are
+// few, else with its whole warp.  Called by whole warps.
+__device__ __forceinline__ void fill_rows(int64_t lo, int64_t hi, int64_t at, int64_t *roff) {
+  const int lane = threadIdx.x & 31;
+  const bool wide = hi - lo > 32;
+  if (!wide)
+    for (int64_t w = lo + 1; w <= hi; ++w) roff[w] = at;
+  for (unsigned m = __ballot_sync(0xffffffffu, wide); m; m &= m - 1) {
+    const int src = __ffs(m) - 1;
+    const int64_t a = __shfl_sync(0xffffffffu, lo, src), b = __shfl_sync(0xffffffffu, hi, src);
+    const int64_t x = __shfl_sync(0xffffffffu, at, src);
+    for (int64_t w = a + 1 + lane; w <= b; w += 32) roff[w] = x;
   }
 }
 
@@ -70,11 +125,16 @@ __global__ void k_arcs_by_tail(const int64_t *off, const int32_t *col, int32_t n
 // first position whose head is >= w.  Position i sets it for the heads w in
 // (key[i-1], key[i]], with key[-1] = -1 and key[nnz] = n, so every w in
 // [0, n] is set exactly once (roff[n] = nnz).
-__global__ void k_in_offsets(const uint32_t *__restrict__ key, int64_t nnz, int32_t n, int64_t *roff) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= nnz; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t lo = i == 0 ? -1 : (int64_t)key[i - 1];
-    const int64_t hi = i == nnz ? (int64_t)n : (int64_t)key[i];
-    for (int64_t w = lo + 1; w <= hi; ++w) roff[w] = i;
+__global__ void __launch_bounds__(256) k_in_offsets(const uint32_t *__restrict__ key, int64_t nnz, int32_t n,
+                                                    int64_t *roff) {
+  const int64_t span = (nnz + 32) & ~(int64_t)31;  // positions 0 .. nnz, in whole warps
+  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < span; i += (int64_t)gridDim.x * 256) {
+    int64_t lo = 0, hi = 0;
+    if (i <= nnz) {
+      lo = i == 0 ? -1 : (int64_t)key[i - 1];
+      hi = i == nnz ? (int64_t)n : (int64_t)key[i];
+    }
+    fill_rows(lo, hi, i, roff);
   }
 }
 
@@ -126,34 +186,99 @@ __global__ void k_check_ids(const int64_t *__restrict__ off, const int32_t *__re
 }
 
 // Arc list of the input rows (u, v), and with `both` also (v, u).
-__global__ void k_arc_list(const int64_t *__restrict__ off, const int32_t *__restrict__ col, int32_t n, int64_t nnz,
-                           bool both, uint32_t *tail, uint32_t *head) {
-  for (int32_t u = blockIdx.x * blockDim.y + threadIdx.y; u < n; u += gridDim.x * blockDim.y)
-    for (int64_t e = off[u] + threadIdx.x; e < off[u + 1]; e += blockDim.x) {
-      tail[e] = (uint32_t)u;
-      head[e] = (uint32_t)col[e];
-      if (both) {
-        tail[nnz + e] = (uint32_t)col[e];
-        head[nnz + e] = (uint32_t)u;
-      }
+__global__ void __launch_bounds__(256) k_arc_list(const int64_t *__restrict__ off, const int32_t *__restrict__ col,
+                                                  int32_t n, int64_t nnz, bool both, uint32_t *tail, uint32_t *head) {
+  for_arcs(off, n, nnz, [&](int64_t e, int32_t u) {
+    const uint32_t v = (uint32_t)col[e];
+    tail[e] = (uint32_t)u;
+    head[e] = v;
+    if (both) {
+      tail[nnz + e] = v;
+      head[nnz + e] = (uint32_t)u;
     }
+  });
 }
 
-// keep[i] = arc i (of the list sorted by (tail, head)) is not a self-loop and
-// not a repeat of arc i - 1; cnt[tail] counts the kept arcs of each row.
-__global__ void k_keep_arcs(const uint32_t *__restrict__ tail, const uint32_t *__restrict__ head, int64_t A,
-                            int64_t *keep, int32_t *cnt) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < A; i += (int64_t)gridDim.x * blockDim.x) {
-    const bool k = tail[i] != head[i] && (i == 0 || tail[i] != tail[i - 1] || head[i] != head[i - 1]);
-    keep[i] = k;
-    if (k) atomicAdd(&cnt[tail[i]], 1);
+// The arcs of the list sorted by (tail, head) that stay (not a self-loop, not a
+// repeat of the arc before) in two passes over tiles of kKeepTile: their number in
+// each tile, then (after a scan of the numbers) their heads in place and the
+// row offsets, which come from the same positions: row w starts at the number
+// of arcs kept before the first arc of a tail >= w.  (Counting rows by atomics
+// waited on the hubs' counters: 0.57 ms for 16.8 million arcs, and flags and
+// positions of 8 bytes an arc went through memory; both passes take 0.10.)
+constexpr int kKeepItems = 8, kKeepTile = 256 * kKeepItems;  // consecutive arcs a thread, and a block
+
+// The thread's arcs (base .. base + kKeepItems - 1) and the one before them;
+// bit i of the result: arc base + i stays.
+__device__ __forceinline__ unsigned keep_load(const uint32_t *__restrict__ tail, const uint32_t *__restrict__ head,
+                                              int64_t A, int64_t base, uint32_t *t, uint32_t *h) {
+  t[0] = base > 0 && base <= A ? tail[base - 1] : 0xFFFFFFFFu;
+  h[0] = base > 0 && base <= A ? head[base - 1] : 0xFFFFFFFFu;
+  if (base + kKeepItems <= A && (((uintptr_t)tail | (uintptr_t)head) & 15) == 0) {
+#pragma unroll
+    for (int i = 0; i < kKeepItems; i += 4) {
+      const uint4 a = *(const uint4 *)(tail + base + i), b = *(const uint4 *)(head + base + i);
+      t[i + 1] = a.x, t[i + 2] = a.y, t[i + 3] = a.z, t[i + 4] = a.w;
+      h[i + 1] = b.x, h[i + 2] = b.y, h[i + 3] = b.z, h[i + 4] = b.w;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < kKeepItems; ++i) {
+      t[i + 1] = base + i < A ? tail[base + i] : 0u;
+      h[i + 1] = base + i < A ? head[base + i] : 0u;
+    }
+  }
+  unsigned k = 0;
+#pragma unroll
+  for (int i = 0; i < kKeepItems; ++i)  // (no arc before the first: its ids are out of range)
+    if (base + i < A && t[i + 1] != h[i + 1] && (t[i + 1] != t[i] || h[i + 1] != h[i])) k |= 1u << i;
+  return k;
+}
+
+__global__ void __launch_bounds__(256) k_keep_count(const uint32_t *__restrict__ tail,
+                                                    const uint32_t *__restrict__ head, int64_t A, int64_t *cnt) {
+  __shared__ uint32_t wc[8];
+  uint32_t t[kKeepItems + 1], h[kKeepItems + 1];
+  const int64_t base = (int64_t)blockIdx.x * kKeepTile + threadIdx.x * kKeepItems;
+  const uint32_t c = __reduce_add_sync(0xffffffffu, (uint32_t)__popc(keep_load(tail, head, A, base, t, h)));
+  if ((threadIdx.x & 31) == 0) wc[threadIdx.x >> 5] = c;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t s = 0;
+    for (int w = 0; w < 8; ++w) s += wc[w];
+    cnt[blockIdx.x] = s;
   }
 }
 
-__global__ void k_pack_arcs(const uint32_t *__restrict__ head, const int64_t *__restrict__ keep,
-                            const int64_t *__restrict__ pos, int64_t A, int32_t *col) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < A; i += (int64_t)gridDim.x * blockDim.x)
-    if (keep[i]) col[pos[i]] = (int32_t)head[i];
+__global__ void __launch_bounds__(256) k_keep_pack(const uint32_t *__restrict__ tail,
+                                                   const uint32_t *__restrict__ head, int64_t A,
+                                                   const int64_t *__restrict__ tile_pos, int32_t n, int32_t *col,
+                                                   int64_t *off) {
+  __shared__ uint32_t wc[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t t[kKeepItems + 1], h[kKeepItems + 1];
+  const int64_t base = (int64_t)blockIdx.x * kKeepTile + threadIdx.x * kKeepItems;
+  const unsigned k = keep_load(tail, head, A, base, t, h);
+  uint32_t inc = (uint32_t)__popc(k);
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) wc[wid] = inc;
+  __syncthreads();
+  int64_t at = tile_pos[blockIdx.x] + (inc - (uint32_t)__popc(k));
+  for (int w = 0; w < wid; ++w) at += wc[w];
+#pragma unroll
+  for (int i = 0; i < kKeepItems; ++i) {
+    // rows that start here: those in (the tail before, this tail], and at position A all that are left
+    int64_t lo = 0, hi = 0;
+    if (base + i <= A) {
+      lo = base + i == 0 ? -1 : (int64_t)t[i];
+      hi = base + i == A ? (int64_t)n : (int64_t)t[i + 1];
+    }
+    if (__any_sync(0xffffffffu, hi > lo)) fill_rows(lo, hi, at, off);
+    if ((k >> i) & 1u) col[at++] = (int32_t)h[i + 1];
+  }
 }
 
 // Canonical CSR of the input rows on the device: rows sorted, repeated arcs and
@@ -189,43 +314,40 @@ void graph_canonicalize(cen_graph *g, const int64_t *off, const int32_t *col, in
     g->nnz = 0;
     return;
   }
-  DevBuf tail, head, k2, v2, hist, tmp, keep, pos, cnt;
+  DevBuf tail, head, k2, v2, hist, tmp, pos;
   tail.ensure(4 * (size_t)A, st);
   head.ensure(4 * (size_t)A, st);
   launch(S, K_GRAPH, st, [&] {
-    k_arc_list<<<grid_for((size_t)n, 8, sm_count() * 64), dim3(32, 8), 0, st>>>(ioff.as<int64_t>(), icol.as<int32_t>(), n,
-                                                                        nnz, symmetrize, tail.as<uint32_t>(),
-                                                                        head.as<uint32_t>());
+    k_arc_list<<<grid_for((size_t)nnz, 8 * kArcRun, sm_count() * 64), 256, 0, st>>>(
+        ioff.as<int64_t>(), icol.as<int32_t>(), n, nnz, symmetrize, tail.as<uint32_t>(), head.as<uint32_t>());
   });
   int bits = 1;
   while (bits < 31 && (1u << bits) < (uint32_t)n) ++bits;
   // by head, then (stably) by tail: the arcs end up sorted by (tail, head)
   radix_sort_pairs(head.as<uint32_t>(), tail.as<uint32_t>(), (size_t)A, bits, k2, v2, hist, tmp, st, S);
   radix_sort_pairs(tail.as<uint32_t>(), head.as<uint32_t>(), (size_t)A, bits, k2, v2, hist, tmp, st, S);
-  keep.ensure(8 * (size_t)A, st);
-  pos.ensure(8 * (size_t)(A + 1), st);
-  cnt.ensure(4 * (size_t)n, st);
-  CEN_CK(cudaMemsetAsync(cnt.p, 0, 4 * (size_t)n, st));
+  // tiles cover positions 0 .. A: position A closes the last rows
+  const int64_t tiles = A / kKeepTile + 1;
+  pos.ensure(8 * (size_t)(tiles + 1), st);
   launch(S, K_GRAPH, st, [&] {
-    k_keep_arcs<<<grid_for((size_t)A, 256), 256, 0, st>>>(tail.as<uint32_t>(), head.as<uint32_t>(), A,
-                                                           keep.as<int64_t>(), cnt.as<int32_t>());
+    k_keep_count<<<(unsigned)tiles, 256, 0, st>>>(tail.as<uint32_t>(), head.as<uint32_t>(), A, pos.as<int64_t>());
   });
-  exclusive_scan_i64(keep.as<int64_t>(), pos.as<int64_t>(), (size_t)A, pos.as<int64_t>() + A, tmp, st, S);
+  exclusive_scan_i64(pos.as<int64_t>(), pos.as<int64_t>(), (size_t)tiles, pos.as<int64_t>() + tiles, tmp, st, S);
   launch(S, K_GRAPH, st, [&] {
-    k_pack_arcs<<<grid_for((size_t)A, 256), 256, 0, st>>>(head.as<uint32_t>(), keep.as<int64_t>(), pos.as<int64_t>(),
-                                                           A, g->col.as<int32_t>());
+    k_keep_pack<<<(unsigned)tiles, 256, 0, st>>>(tail.as<uint32_t>(), head.as<uint32_t>(), A, pos.as<int64_t>(), n,
+                                                 g->col.as<int32_t>(), g->off.as<int64_t>());
   });
-  counts_to_offsets(cnt.as<int32_t>(), g->off.as<int64_t>(), (size_t)n, tmp, st, S);
   int64_t kept = 0;
-  CEN_CK(cudaMemcpyAsync(&kept, pos.as<int64_t>() + A, 8, cudaMemcpyDeviceToHost, st));
+  CEN_CK(cudaMemcpyAsync(&kept, pos.as<int64_t>() + tiles, 8, cudaMemcpyDeviceToHost, st));
   CEN_CK(cudaStreamSynchronize(st));
   g->nnz = kept;
 }
 
-// Sums of d and d^2 over the rows of off (one pass, double sums).
-__global__ void k_degree_moments(const int64_t *__restrict__ off, int32_t n, double *sums) {
+// Sums of d and d^2 over the rows of off (one pass, double sums, two atomics a block).
+__global__ void __launch_bounds__(256) k_degree_moments(const int64_t *__restrict__ off, int32_t n, double *sums) {
+  __shared__ double sa[8], sb[8];
   double a = 0.0, b = 0.0;
-  for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+  for (int64_t v = (int64_t)blockIdx.x * 256 + threadIdx.x; v < n; v += (int64_t)gridDim.x * 256) {
     const double d = (double)(off[v + 1] - off[v]);
     a += d;
     b += d * d;
@@ -233,6 +355,15 @@ __global__ void k_degree_moments(const int64_t *__restrict__ off, int32_t n, dou
   a = warp_sum(a);
   b = warp_sum(b);
   if ((threadIdx.x & 31) == 0) {
+    sa[threadIdx.x >> 5] = a;
+    sb[threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) {
+      a += sa[w];
+      b += sb[w];
+    }
     atomicAdd(&sums[0], a);
     atomicAdd(&sums[1], b);
   }
@@ -340,8 +471,8 @@ void graph_build(cen_graph *g, const int64_t *off, const int32_t *col, bool on_d
   key.ensure(4 * (size_t)nnz, st);
   g->rcol.ensure(4 * (size_t)nnz, st);
   launch(S, K_GRAPH, st, [&] {
-    k_arcs_by_tail<<<grid_for((size_t)n, 8), 256, 0, st>>>(g->off.as<int64_t>(), g->col.as<int32_t>(), n,
-                                                           key.as<uint32_t>(), g->rcol.as<uint32_t>());
+    k_arcs_by_tail<<<grid_for((size_t)nnz, 8 * kArcRun, sm_count() * 64), 256, 0, st>>>(
+        g->off.as<int64_t>(), g->col.as<int32_t>(), n, nnz, key.as<uint32_t>(), g->rcol.as<uint32_t>());
   });
   int bits = 1;
   while (bits < 31 && (1u << bits) < (uint32_t)n) ++bits;
