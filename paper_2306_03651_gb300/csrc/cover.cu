@@ -14,46 +14,106 @@ namespace cg = cooperative_groups;
 namespace cen {
 
 // ------------------------------------------------------- incidence
-__global__ void k_count_members(const int32_t *__restrict__ hmem, int64_t total, int32_t *c) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&c[hmem[i]], 1);
+constexpr int kRankThreads = 512;
+// Members from which a thread takes eight, below it two (more blocks); the time
+// of all rounds of a run, two against eight: BA n = 2,000 up to 0.6M members
+// 75 and 81 us, R-MAT 18 up to 3M members 165 and 120 us.
+constexpr size_t kRankWide = (size_t)1 << 19;
+
+// Counts every node's members in c (zero before) and gives each member its
+// place among its node's (in no particular order).  A block's members meet in
+// a table of as many slots in shared memory, and each node found there takes
+// one atomic on its count for the whole block; a node that finds no slot within
+// kRankProbes takes one per member.  The counts of hub nodes are what bounds
+// this: with one atomic a member to count it and another to place it, all on a
+// few addresses at L2, a run's rounds took 256 + 225 us on BA n = 2,000 (0.6M
+// members at the end) and 489 + 511 us on R-MAT 18 (3M); they take 75 + 29 and
+// 120 + 66.
+constexpr int kRankProbes = 4;
+template <int ITEMS>
+__global__ void __launch_bounds__(kRankThreads) k_rank_members(const int32_t *__restrict__ hmem, int64_t total,
+                                                               int32_t *c, int32_t *__restrict__ rank) {
+  constexpr int TILE = kRankThreads * ITEMS;
+  static_assert(TILE <= 4096 && (TILE & (TILE - 1)) == 0, "12-bit slots and places");
+  __shared__ int32_t key[TILE], cnt[TILE];
+  for (int p = threadIdx.x; p < TILE; p += kRankThreads) {
+    key[p] = -1;
+    cnt[p] = 0;
+  }
+  __syncthreads();
+  const int64_t base = (int64_t)blockIdx.x * TILE + threadIdx.x;
+  uint32_t at[ITEMS];  // slot << 16 | place among the block's members of the node
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const int64_t i = base + r * kRankThreads;
+    at[r] = ~0u;
+    if (i >= total) continue;
+    const int32_t u = hmem[i];
+    uint32_t p = ((uint32_t)u * 0x9E3779B1u) >> 20 & (TILE - 1);
+    bool found = false;
+    for (int k = 0; k < kRankProbes && !found; ++k) {
+      int32_t have = *(volatile int32_t *)&key[p];
+      if (have == -1) have = atomicCAS(&key[p], -1, u);
+      found = have == -1 || have == u;
+      if (!found) p = (p + 1) & (TILE - 1);
+    }
+    if (found)
+      at[r] = (p << 16) | (uint32_t)atomicAdd(&cnt[p], 1);
+    else
+      rank[i] = atomicAdd(&c[u], 1);
+  }
+  __syncthreads();
+  for (int p = threadIdx.x; p < TILE; p += kRankThreads)
+    if (key[p] >= 0) cnt[p] = atomicAdd(&c[key[p]], cnt[p]);
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r)
+    if (at[r] != ~0u) rank[base + r * kRankThreads] = cnt[at[r] >> 16] + (int32_t)(at[r] & 0xFFFFu);
 }
 
-// Thread per sample: each member u gets j appended to row u (order within a
-// row follows atomic arrival; every consumer of the rows is order-free).
-__global__ void k_scatter_members(const int64_t *__restrict__ hoff, const int32_t *__restrict__ hmem, uint64_t m,
-                                  const int64_t *__restrict__ noff, int32_t *cursor, int32_t *nsamp) {
-  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (uint64_t)gridDim.x * blockDim.x) {
-    for (int64_t e = hoff[j]; e < hoff[j + 1]; ++e) {
-      const int32_t u = hmem[e];
-      const int32_t pos = atomicAdd(&cursor[u], 1);
-      nsamp[noff[u] + pos] = (int32_t)j;
-    }
+// GS lanes per sample: each member u gets j at its place of row u (the order
+// within a row is free; every consumer of the rows is order-free).
+template <int GS>
+__global__ void k_place_members(const int64_t *__restrict__ hoff, const int32_t *__restrict__ hmem, uint64_t m,
+                                const int64_t *__restrict__ noff, const int32_t *__restrict__ rank, int32_t *nsamp) {
+  const int lane = threadIdx.x & (GS - 1);
+  const uint64_t groups = (uint64_t)gridDim.x * blockDim.x / GS;
+  for (uint64_t j = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / GS; j < m; j += groups) {
+    const int64_t e1 = hoff[j + 1];
+    for (int64_t e = hoff[j] + lane; e < e1; e += GS) nsamp[noff[hmem[e]] + rank[e]] = (int32_t)j;
   }
 }
 
+// Rows of the samples that hold each node.  The members' places lie in hmemh,
+// which build_heavy fills anew afterwards.
 void build_incidence(cen_job *job) {
   if (job->inc_m == job->m) return;
   cudaStream_t st = job->st;
   Stats *S = &job->stats;
   const int32_t n = job->g->n;
+  const size_t members = (size_t)job->members;
   job->c.ensure(4 * (size_t)n, st);
-  job->cursor.ensure(4 * (size_t)n, st);
   job->noff.ensure(8 * ((size_t)n + 1), st);
-  job->nsamp.ensure(4 * (size_t)(job->members + 1), st);
+  job->nsamp.ensure(4 * (members + 1), st);
+  job->hmemh.ensure(4 * (members + 1), st);
+  job->heavy_m = ~0ull;
   CEN_CK(cudaMemsetAsync(job->c.p, 0, 4 * (size_t)n, st));
-  CEN_CK(cudaMemsetAsync(job->cursor.p, 0, 4 * (size_t)n, st));
-  if (job->members)
+  if (members)
     launch(S, K_TRANSPOSE, st, [&] {
-      k_count_members<<<grid_for((size_t)job->members, 256), 256, 0, st>>>(job->hmem.as<int32_t>(), job->members,
-                                                                         job->c.as<int32_t>());
+      const bool wide = members >= kRankWide;
+      auto kernel = wide ? k_rank_members<8> : k_rank_members<2>;
+      const int tile = kRankThreads * (wide ? 8 : 2);
+      kernel<<<(unsigned)((members + tile - 1) / tile), kRankThreads, 0, st>>>(
+          job->hmem.as<int32_t>(), job->members, job->c.as<int32_t>(), job->hmemh.as<int32_t>());
     });
   counts_to_offsets(job->c.as<int32_t>(), job->noff.as<int64_t>(), (size_t)n, job->scan_tmp, st, S);
-  if (job->m)
+  if (members)
     launch(S, K_TRANSPOSE, st, [&] {
-      k_scatter_members<<<grid_for(job->m, 256), 256, 0, st>>>(job->hoff.as<int64_t>(), job->hmem.as<int32_t>(),
-                                                               job->m, job->noff.as<int64_t>(),
-                                                               job->cursor.as<int32_t>(), job->nsamp.as<int32_t>());
+      const bool wide = job->members > kShortMembers * (int64_t)job->m;
+      auto kernel = wide ? k_place_members<32> : k_place_members<4>;
+      kernel<<<grid_for(job->m * (wide ? 32 : 4), 256), 256, 0, st>>>(
+          job->hoff.as<int64_t>(), job->hmem.as<int32_t>(), job->m, job->noff.as<int64_t>(),
+          job->hmemh.as<int32_t>(), job->nsamp.as<int32_t>());
     });
   job->inc_m = job->m;
 }

@@ -26,7 +26,7 @@ struct WaveWS {
   DevBuf ctl;                                 // control block (see sampler.cu)
   DevBuf jlist;                               // explicit sample ids for a re-run
   DevBuf woff;                                // wave-local member offsets per slot
-  DevBuf lens, exoff, scan_tmp;               // offsets of appended samples (workspace 0)
+  DevBuf scan_tmp;                            // offsets of appended samples (workspace 0)
   void *host = nullptr;                       // pinned staging for this pipeline
   size_t host_bytes = 0;
   cudaStream_t own_stream = nullptr;          // stream of an extra pipeline (null for the job's)
@@ -35,8 +35,8 @@ struct WaveWS {
   ~WaveWS() {
     if (own_stream) {
       cudaStreamSynchronize(own_stream);
-      for (DevBuf *b : {&vis, &lev_ptrs, &tmp, &any, &base, &cnt, &sigc, &ovf, &slots, &ctl, &jlist, &woff, &lens,
-                        &exoff, &scan_tmp, &arcs, &arc_range})
+      for (DevBuf *b : {&vis, &lev_ptrs, &tmp, &any, &base, &cnt, &sigc, &ovf, &slots, &ctl, &jlist, &woff,
+                        &scan_tmp, &arcs, &arc_range})
         b->st = nullptr;
       for (auto &l : lev) l->st = nullptr;
     }
@@ -130,7 +130,7 @@ struct cen_job {
   // sample store (device): hoff[m+1], hmem[members], per-sample s, t, d, sign words
   cen::DevBuf hoff, hmem, ps, pt, pd, sign, bmax;
   // node -> sample incidence (rebuilt lazily when m changed)
-  cen::DevBuf c, noff, nsamp, cursor;
+  cen::DevBuf c, noff, nsamp;
   uint64_t inc_m = ~0ull;
   // heavy nodes of the sample (heavy.cuh) and whether the last greedy / AMCERA needed all nodes
   cen::DevBuf hctl, hlist, hc, hidx, hchunks, hmemh;
@@ -175,6 +175,8 @@ struct cen_job {
 };
 
 namespace cen {
+// Samples of more members than this on average are moved by a warp each, others by four lanes.
+constexpr int64_t kShortMembers = 16;
 void sample_append(cen_job *job, uint64_t m_new);
 void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages);
 void bidir_launch_rest(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages, uint64_t left);

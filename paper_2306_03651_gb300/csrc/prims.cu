@@ -10,7 +10,7 @@
 #include <mutex>
 #include <vector>
 
-#include "common.cuh"
+#include "scan.cuh"
 
 namespace cen {
 
@@ -182,95 +182,13 @@ void allow_shared(const void *kernel, size_t bytes) {
 }
 
 // -------------------------------------------------------------- scans
-constexpr int kScanThreads = 1024, kScanItems = 4, kScanTile = kScanThreads * kScanItems;
-
-template <class T>
-__device__ __forceinline__ T block_exclusive_scan(T v, T *smem_warp, T *total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    T y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) smem_warp[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    T w = (lane < (int)(blockDim.x >> 5)) ? smem_warp[lane] : T(0);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      T y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
-    }
-    if (lane < (int)(blockDim.x >> 5)) smem_warp[lane] = w;  // inclusive warp totals
-  }
-  __syncthreads();
-  T before = warp ? smem_warp[warp - 1] : T(0);
-  *total = smem_warp[(blockDim.x >> 5) - 1];
-  __syncthreads();
-  return before + x - v;
-}
-
-template <class T>
-__global__ void scan_partials(const T *in, size_t n, T *part) {
-  __shared__ T sw[32];
-  size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
-  T s = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i)
-    if (base + i < n) s += in[base + i];
-  T tot;
-  block_exclusive_scan<T>(s, sw, &tot);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
-template <class T>
-__global__ void scan_top(T *part, size_t nparts, T *d_total) {
-  __shared__ T sw[32];
-  T carry = 0;
-  for (size_t base = 0; base < nparts; base += blockDim.x) {
-    size_t i = base + threadIdx.x;
-    T v = i < nparts ? part[i] : T(0);
-    T tot;
-    T ex = block_exclusive_scan<T>(v, sw, &tot);
-    if (i < nparts) part[i] = carry + ex;
-    carry += tot;
-  }
-  if (threadIdx.x == 0 && d_total) *d_total = carry;
-}
-
-template <class T>
-__global__ void scan_final(const T *in, T *out, size_t n, const T *part) {
-  __shared__ T sw[32];
-  size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanItems;
-  T v[kScanItems];
-  T s = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    v[i] = (base + i < n) ? in[base + i] : T(0);
-    s += v[i];
-  }
-  T tot;
-  T ex = block_exclusive_scan<T>(s, sw, &tot) + part[blockIdx.x];
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    if (base + i < n) out[base + i] = ex;
-    ex += v[i];
-  }
-}
-
 template <class T>
 static void exclusive_scan(const T *in, T *out, size_t n, T *d_total, DevBuf &tmp, cudaStream_t st, Stats *S) {
   if (n == 0) {
     if (d_total) CEN_CK(cudaMemsetAsync(d_total, 0, sizeof(T), st));
     return;
   }
-  size_t nparts = (n + kScanTile - 1) / kScanTile;
-  tmp.ensure(nparts * sizeof(T), st);
-  T *part = tmp.as<T>();
-  launch(S, K_MISC, st, [&] { scan_partials<T><<<(unsigned)nparts, kScanThreads, 0, st>>>(in, n, part); });
-  launch(S, K_MISC, st, [&] { scan_top<T><<<1, kScanThreads, 0, st>>>(part, nparts, d_total); });
-  launch(S, K_MISC, st, [&] { scan_final<T><<<(unsigned)nparts, kScanThreads, 0, st>>>(in, out, n, part); });
+  device_scan<T>(ScanArray<T, T>{in}, ScanOffsets<T>{out, d_total, n}, n, tmp, st, S);
 }
 
 void exclusive_scan_i64(const int64_t *in, int64_t *out, size_t n, int64_t *d_total, DevBuf &tmp, cudaStream_t st,
@@ -278,14 +196,12 @@ void exclusive_scan_i64(const int64_t *in, int64_t *out, size_t n, int64_t *d_to
   exclusive_scan<int64_t>(in, out, n, d_total, tmp, st, S);
 }
 
-__global__ void widen_i32(const int32_t *cnt, int64_t *out, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = cnt[i];
-}
-
 void counts_to_offsets(const int32_t *cnt, int64_t *out, size_t n, DevBuf &tmp, cudaStream_t st, Stats *S) {
-  if (n) launch(S, K_MISC, st, [&] { widen_i32<<<grid_for(n, 256), 256, 0, st>>>(cnt, out, n); });
-  exclusive_scan<int64_t>(out, out, n, out + n, tmp, st, S);
+  if (n == 0) {
+    CEN_CK(cudaMemsetAsync(out, 0, sizeof(int64_t), st));
+    return;
+  }
+  device_scan<int64_t>(ScanArray<int64_t, int32_t>{cnt}, ScanOffsets<int64_t>{out, out + n, n}, n, tmp, st, S);
 }
 
 // --------------------------------------------------------- radix sort

@@ -30,6 +30,7 @@
 #include <thread>
 
 #include "job.cuh"
+#include "scan.cuh"
 
 namespace cen {
 
@@ -421,33 +422,32 @@ __global__ void __launch_bounds__(1024) k_wave_lengths(int count, uint64_t jbase
   if (threadIdx.x == 0) ctl->total = carry;
 }
 
-// Member counts of samples j0 .. j0+count-1 from their third field: set
-// betweenness max(d - 1, 0) (the interior of a d-arc path), kappa-path the
-// steps taken, triangle 3.
-__global__ void k_lengths_of(const int32_t *__restrict__ pd, uint64_t j0, uint64_t count, int space, int32_t *lens) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (uint64_t)gridDim.x * blockDim.x) {
-    const int d = pd[j0 + i];
-    lens[i] = space == CEN_SPACE_KPATH ? d : space == CEN_SPACE_TRIANGLE ? 3 : (d >= 2 ? d - 1 : 0);
+// Member count of a new sample from its third field: betweenness
+// max(d - 1, 0) (the interior of a d-arc path), kappa-path the steps taken,
+// triangle 3.
+struct SampleLength {
+  const int32_t *pd;  // of the new samples
+  int space;
+  __device__ int64_t operator()(size_t i) const {
+    const int d = pd[i];
+    return space == CEN_SPACE_KPATH ? d : space == CEN_SPACE_TRIANGLE ? 3 : (d >= 2 ? d - 1 : 0);
   }
-}
+};
+struct SampleEnd {
+  int64_t *hoff;  // of the first new sample
+  __device__ void operator()(size_t i, int64_t before, int64_t len) const { hoff[i + 1] = hoff[0] + before + len; }
+};
 
-// Warp per new sample: lens[i] members from src[i * stride] to the store.
-__global__ void k_gather_strided(uint64_t count, uint64_t j0, int stride, const int32_t *__restrict__ lens,
-                                 const int64_t *__restrict__ hoff, const int32_t *__restrict__ src, int32_t *hmem) {
+// Warp per new sample: its members from src[i * stride] to the store.
+__global__ void k_gather_strided(uint64_t count, uint64_t j0, int stride, const int64_t *__restrict__ hoff,
+                                 const int32_t *__restrict__ src, int32_t *hmem) {
   const int lane = threadIdx.x & 31;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < count; i += nwarps) {
     const int64_t h = hoff[j0 + i];
-    for (int q = lane; q < lens[i]; q += 32) hmem[h + q] = src[i * (uint64_t)stride + q];
+    const int len = (int)(hoff[j0 + i + 1] - h);
+    for (int q = lane; q < len; q += 32) hmem[h + q] = src[i * (uint64_t)stride + q];
   }
-}
-
-// hoff[j0 + i] = hoff[j0] + ex[i] for i = 1 .. count.
-__global__ void k_hoff_add(int64_t *hoff, uint64_t j0, uint64_t count, const int64_t *__restrict__ ex) {
-  const int64_t base = hoff[j0];
-  for (uint64_t i = 1 + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= count;
-       i += (uint64_t)gridDim.x * blockDim.x)
-    hoff[j0 + i] = base + ex[i];
 }
 
 // aoff[jlist[b] - j0] = base + woff[b] for the slots of a wave whose members
@@ -458,18 +458,20 @@ __global__ void k_set_aoff(int count, const uint64_t *__restrict__ jlist, uint64
     aoff[jlist[b] - j0] = slot_d[b] >= 2 ? base + woff[b] : -1;
 }
 
-// Warp per new sample: its members move from the arena (at aoff) to the store.
+// Members of the new samples move from the arena (at aoff) to the store, by GS
+// lanes a sample.
+template <int GS>
 __global__ void k_gather_arena(uint64_t count, uint64_t j0, const int64_t *__restrict__ aoff,
                                const int32_t *__restrict__ pd, const int64_t *__restrict__ hoff,
                                const int32_t *__restrict__ arena, int32_t *hmem) {
-  const int lane = threadIdx.x & 31;
-  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < count; i += nwarps) {
+  const int lane = threadIdx.x & (GS - 1);
+  const uint64_t groups = (uint64_t)gridDim.x * blockDim.x / GS;
+  for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / GS; i < count; i += groups) {
     const int64_t a = aoff[i];
     const int d = pd[j0 + i];
     if (a < 0 || d < 2) continue;
     const int64_t h = hoff[j0 + i];
-    for (int q = lane; q < d - 1; q += 32) hmem[h + q] = arena[a + q];
+    for (int q = lane; q < d - 1; q += GS) hmem[h + q] = arena[a + q];
   }
 }
 
@@ -1259,27 +1261,18 @@ void rerun_in_place(cen_job *job, std::vector<uint64_t> ids) {
   }
 }
 
-// hoff of the new samples from their distances; returns their member total
-// (known_total, when the caller has counted it, saves reading it back).
+// hoff of the new samples from their distances (one scan over the lengths,
+// which follow from the distances); returns their member total (known_total,
+// when the caller knows it, saves reading it back).
 int64_t offsets_from_distances(cen_job *job, uint64_t m0, uint64_t m_new, int64_t known_total = -1) {
   cudaStream_t st = job->st;
-  Stats *S = &job->stats;
-  WaveWS &w0 = wave_ws0(job);
-  w0.lens.ensure(4 * (size_t)m_new, st);
-  w0.exoff.ensure(8 * ((size_t)m_new + 1), st);
-  launch(S, K_APPEND, st, [&] {
-    k_lengths_of<<<grid_for(m_new, 256), 256, 0, st>>>(job->pd.as<int32_t>(), m0, m_new, job->space,
-                                                        w0.lens.as<int32_t>());
-  });
-  counts_to_offsets(w0.lens.as<int32_t>(), w0.exoff.as<int64_t>(), (size_t)m_new, w0.scan_tmp, st, S);
-  launch(S, K_APPEND, st, [&] {
-    k_hoff_add<<<grid_for(m_new, 256), 256, 0, st>>>(job->hoff.as<int64_t>(), m0, m_new, w0.exoff.as<int64_t>());
-  });
-  if (known_total >= 0) return known_total;  // the caller counted the members already
+  device_scan<int64_t>(SampleLength{job->pd.as<int32_t>() + m0, job->space}, SampleEnd{job->hoff.as<int64_t>() + m0},
+                       (size_t)m_new, wave_ws0(job).scan_tmp, st, &job->stats, K_APPEND);
+  if (known_total >= 0) return known_total;
   int64_t *h = (int64_t *)host_staging(job, 8);
-  CEN_CK(cudaMemcpyAsync(h, w0.exoff.as<int64_t>() + m_new, 8, cudaMemcpyDeviceToHost, st));
+  CEN_CK(cudaMemcpyAsync(h, job->hoff.as<int64_t>() + m0 + m_new, 8, cudaMemcpyDeviceToHost, st));
   CEN_CK(cudaStreamSynchronize(st));
-  return *h;
+  return *h - job->members;
 }
 
 // Workspace for as many resident CTAs as the byte budget allows (at least
@@ -1464,9 +1457,12 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   const int64_t total = offsets_from_distances(job, m0, m_new, search.empty() ? (int64_t)h.cursor : -1);
   job->hmem.ensure(4 * (size_t)(job->members + total + 1), st, 4 * (size_t)job->members);
   launch(&job->stats, K_APPEND, st, [&] {
-    k_gather_arena<<<grid_for(m_new * 32, 256), 256, 0, st>>>(m_new, m0, bw.aoff.as<int64_t>(),
-                                                              job->pd.as<int32_t>(), job->hoff.as<int64_t>(),
-                                                              bw.arena.as<int32_t>(), job->hmem.as<int32_t>());
+    const bool wide = total > kShortMembers * (int64_t)m_new;
+    const int lanes = wide ? 32 : 4;
+    auto kernel = wide ? k_gather_arena<32> : k_gather_arena<4>;
+    kernel<<<grid_for(m_new * lanes, 256), 256, 0, st>>>(m_new, m0, bw.aoff.as<int64_t>(), job->pd.as<int32_t>(),
+                                                         job->hoff.as<int64_t>(), bw.arena.as<int32_t>(),
+                                                         job->hmem.as<int32_t>());
   });
   // walks the CTAs left (cone or counts too large, arena full) and the pairs
   // whose count reached 2^64 in the waves above: written in place
@@ -1499,10 +1495,9 @@ int64_t append_kpath(cen_job *job, uint64_t m0, uint64_t m_new) {
     kpath_sample(job, m0, m_new, job->hmem.as<int32_t>(), job->hoff.as<int64_t>());
     return total;
   }
-  WaveWS &w0 = wave_ws0(job);
   launch(&job->stats, K_APPEND, st, [&] {
-    k_gather_strided<<<grid_for(m_new * 32, 256), 256, 0, st>>>(m_new, m0, job->kappa, w0.lens.as<int32_t>(),
-                                                                job->hoff.as<int64_t>(), job->space_buf.as<int32_t>(),
+    k_gather_strided<<<grid_for(m_new * 32, 256), 256, 0, st>>>(m_new, m0, job->kappa, job->hoff.as<int64_t>(),
+                                                                job->space_buf.as<int32_t>(),
                                                                 job->hmem.as<int32_t>());
   });
   return total;
@@ -1511,7 +1506,7 @@ int64_t append_kpath(cen_job *job, uint64_t m0, uint64_t m_new) {
 // Triangle space: three members each, written in place.
 int64_t append_triangle(cen_job *job, uint64_t m0, uint64_t m_new) {
   cudaStream_t st = job->st;
-  const int64_t total = offsets_from_distances(job, m0, m_new);
+  const int64_t total = offsets_from_distances(job, m0, m_new, 3 * (int64_t)m_new);
   job->hmem.ensure(4 * (size_t)(job->members + total + 1), st, 4 * (size_t)job->members);
   triangle_sample(job, m0, m_new);
   int *h = (int *)host_staging(job, 4);  // |h| = 3 for every sample

@@ -71,8 +71,8 @@ def estimate_job_bytes(n: int, nnz: int, t: int, m_cap: int, avg_hyperedge: floa
     as many as fit in `bidir_budget`.  Wave workspace (the fallback): `levels` + 6 arrays
     of n*G words (G = wave words, at most 32 and at most 1 GB per array) and the
     initial cone-arc log (2 n G records of 24 bytes); sample store for m_cap
-    samples: offsets, endpoints, distance, sign words and members (twice: samples
-    and the incidence), plus the member arena; AMCERA table R[t+1][n] and greedy /
+    samples: offsets, endpoints, distance, sign words and members (samples, incidence
+    and their places in it), plus the member arena; AMCERA table R[t+1][n] and greedy /
     incidence arrays.  `resident_ctas` is the sampler's CTAs in flight (16 per SM
     on a 152-SM GB300)."""
     qc = max(16, min(n, bidir_queue))
@@ -87,7 +87,7 @@ def estimate_job_bytes(n: int, nnz: int, t: int, m_cap: int, avg_hyperedge: floa
     words = n * G
     wave = 8 * words * (levels + 6) + 24 * 2 * words
     nw = (t + 31) // 32
-    store = m_cap * (8 + 12 + 4 * nw) + 3 * 4 * int(m_cap * avg_hyperedge)
+    store = m_cap * (8 + 12 + 4 * nw) + 4 * 4 * int(m_cap * avg_hyperedge)
     node = n * (4 * (t + 1) + 4 * 4 + 8)
     return int(bidir + wave + store + node)
 
