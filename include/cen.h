@@ -391,7 +391,8 @@ int cen_release_cached(void);
  * left whole to the bit-parallel sampler (*deferred_search), samples whose walk
  * it left to it (*deferred_walk), searches that outgrew the small node table
  * or the shared memory of a wide CTA (*migrated), the CTAs (slots) the
- * bidirectional search has global workspace for (0 before its first use), and
+ * bidirectional search may have global workspace for (0 before its first use;
+ * it is allocated when a search needs it), and
  * the warp searches handed on to whole CTAs because a level, the node count or
  * the depth was too large for one warp (*escalated).
  * Any pointer may be NULL. */

@@ -1282,6 +1282,38 @@ static void next_stage(cen_job *job, BiArgs &a, int stage) {
   a.out_count = &ctl->nout[stage];
 }
 
+// Gives `want` CTAs (at most the budget's) their tables in global memory, where
+// fewer have them.  Searches in shared memory need none, and the few that they
+// hand on need them for a CTA per SM at most, so the tables of every CTA in
+// flight (14 GB for graphs of 65,536 nodes or more) are made only for launches
+// that search there with all of them: the first R-MAT 16 round of a process
+// took 17.5 ms, 13 of them to map and clear those, and takes 4.8.
+static int bidir_tables(cen_job *job, uint64_t want) {
+  BiWS &w = *job->bws;
+  cudaStream_t st = job->st;
+  const int slots = (int)std::min<uint64_t>((uint64_t)w.nslots, want);
+  if (w.tables >= slots) return slots;
+  w.tables = 0;
+  const size_t k = (size_t)slots;
+  if (w.H1) w.tab1.ensure_exact(8 * (size_t)w.H1 * k, st);
+  w.tab2.ensure_exact(8 * (size_t)w.H2 * k, st);
+  w.lists.ensure_exact(4 * 7 * (size_t)w.QC * k, st);
+  w.sig.ensure_exact(8 * (size_t)w.H2 * k, st);
+  w.epochs.ensure(8 * k, st);
+  if (w.H1) CEN_CK(cudaMemsetAsync(w.tab1.p, 0, 8 * (size_t)w.H1 * k, st));
+  CEN_CK(cudaMemsetAsync(w.tab2.p, 0, 8 * (size_t)w.H2 * k, st));
+  CEN_CK(cudaMemsetAsync(w.epochs.p, 0, 8 * k, st));
+  if (w.WQ) {
+    const size_t tb = bidir_warp_table_bytes_per_slot() * k, eb = bidir_warp_epoch_bytes_per_slot() * k;
+    w.tabw.ensure_exact(tb, st);
+    w.epw.ensure_exact(eb, st);
+    CEN_CK(cudaMemsetAsync(w.tabw.p, 0, tb, st));
+    CEN_CK(cudaMemsetAsync(w.epw.p, 0, eb, st));
+  }
+  w.tables = slots;
+  return slots;
+}
+
 // Searches every sample of the call; what is left after the launches made here
 // (none after a launch with the tables in global memory) is listed, its number
 // in ctl->nout[*stages - 1].
@@ -1289,6 +1321,7 @@ void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, 
   BiWS &w = *job->bws;
   cudaStream_t st = job->st;
   CEN_CK(cudaMemsetAsync(w.ctl.p, 0, sizeof(BiCtl), st));
+  if (w.WQ || w.tier == kTierGlobal) bidir_tables(job, (uint64_t)w.nslots);
   BiArgs a = bidir_args(job, j0, count, arena_cap);
   const int grid = (int)std::min<uint64_t>((uint64_t)w.nslots, count);
   int stage = 0;
@@ -1325,6 +1358,8 @@ void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, 
 void bidir_launch_rest(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages, uint64_t left) {
   BiWS &w = *job->bws;
   cudaStream_t st = job->st;
+  const int ctas = bidir_tables(job, left < kWideMost ? (uint64_t)sm_count() : (uint64_t)w.nslots);
+  const int grid = (int)std::min<uint64_t>((uint64_t)ctas, left);
   BiArgs a = bidir_args(job, j0, count, arena_cap);
   int stage = *stages;
   next_stage(job, a, stage - 1);
@@ -1332,10 +1367,8 @@ void bidir_launch_rest(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_
   if (left < kWideMost) {
     log_launch<LogHuge>(job, a, left);
     next_stage(job, a, stage++);
-    const int grid = (int)std::min<uint64_t>(std::min<uint64_t>((uint64_t)w.nslots, left), (uint64_t)sm_count());
     launch(&job->stats, K_BIDIR, st, [&] { k_bidir_wide<<<grid, kWideThreads, 0, st>>>(a); });
   } else {
-    const int grid = (int)std::min<uint64_t>((uint64_t)w.nslots, left);
     launch(&job->stats, K_BIDIR, st, [&] { k_bidir<true><<<grid, kBiThreads, 0, st>>>(a); });
   }
   *stages = stage;

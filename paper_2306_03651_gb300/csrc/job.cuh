@@ -48,8 +48,9 @@ struct WaveWS {
   DevBuf arc_range;                           // per level: [first, end) of its logged arcs
 };
 
-// Workspace of the bidirectional sampler (bidir.cu): for each of `nslots`
-// resident CTAs, a small table of H1 entries (0: none) and a large one of H2
+// Workspace of the bidirectional sampler (bidir.cu): the lists of one call's
+// samples and, for each of up to `nslots` resident CTAs that search in global
+// memory, a small table of H1 entries (0: none) and a large one of H2
 // = 4 QC entries, zeroed once (entries are epoch-stamped, so nothing is
 // cleared between samples), seven lists of QC entries (two ball queues, two
 // cone lists, heavy rows, crossing-arc tails and heads) and H2 path counts.
@@ -74,7 +75,8 @@ struct BiWS {
   DevBuf tabw, epw;        // warp searches: node tables and epochs (none when WQ = 0)
   DevBuf big, far;         // ids that a launch hands on to the next (used in turn)
   int tier = 0;            // where searches by CTAs start (kTier*)
-  int nslots = 0;
+  int nslots = 0;          // CTAs that the budget allows tables in global memory for
+  int tables = 0;          // CTAs that have them (bidir_tables)
   int64_t QC = 0;
   int64_t H1 = 0;
   int64_t H2 = 0;

@@ -1327,22 +1327,6 @@ void bidir_setup(cen_job *job, uint64_t m_new) {
   BiWS &wk = *job->bws;
   if (wk.nslots == 0) {
     keep_pool_memory();
-    if (H1) wk.tab1.ensure_exact(8 * (size_t)H1 * slots, st);
-    wk.tab2.ensure_exact(8 * (size_t)H2 * slots, st);
-    wk.lists.ensure_exact(4 * 7 * (size_t)QC * slots, st);
-    wk.sig.ensure_exact(8 * (size_t)H2 * slots, st);
-    wk.epochs.ensure(8 * (size_t)slots, st);
-    if (H1) CEN_CK(cudaMemsetAsync(wk.tab1.p, 0, 8 * (size_t)H1 * slots, st));
-    CEN_CK(cudaMemsetAsync(wk.tab2.p, 0, 8 * (size_t)H2 * slots, st));
-    CEN_CK(cudaMemsetAsync(wk.epochs.p, 0, 8 * (size_t)slots, st));
-    if (WQ) {
-      const size_t tb = bidir_warp_table_bytes_per_slot() * (size_t)slots;
-      const size_t eb = bidir_warp_epoch_bytes_per_slot() * (size_t)slots;
-      wk.tabw.ensure_exact(tb, st);
-      wk.epw.ensure_exact(eb, st);
-      CEN_CK(cudaMemsetAsync(wk.tabw.p, 0, tb, st));
-      CEN_CK(cudaMemsetAsync(wk.epw.p, 0, eb, st));
-    }
     wk.QC = QC;
     wk.WQ = WQ;
     wk.H1 = H1;
