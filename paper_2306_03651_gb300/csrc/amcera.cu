@@ -475,6 +475,14 @@ static void mcera_over_all(cen_job *job, int32_t k, void *h, int64_t *Rnum, int6
   CEN_REQUIRE(mcera_result(job, k, h, Rnum, Wnum, b), CEN_ECUDA, "cen_mcera: the select left a row open");
 }
 
+// The first such call of a job that has at most this many sign words to read
+// (members x words) runs the AMCERA ahead of greedyCover on the job's stream:
+// its 10 us are less than the 20 a second stream takes to make and give back,
+// and many jobs make one call (BA 2,000, 50,000 members: a round's 222 us
+// instead of 235).  A job that calls again makes the second stream: without
+// it, the nine rounds of a certified run on that graph take 4.25 ms, not 4.11.
+constexpr uint64_t kAsideWords = (uint64_t)1 << 17;
+
 // greedyCover on the job's stream and the AMCERA on its second stream at the
 // same time: the two read the same incidence and write disjoint buffers, so
 // the results are those of greedy_cover followed by mcera.
@@ -488,6 +496,16 @@ void cover_and_mcera(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint6
   mcera_prepare(job, k);
   const size_t gb = (greedy_result_bytes(k) + 15) & ~(size_t)15;
   char *h = (char *)host_staging(job, gb + mcera_result_bytes(job));
+  if (!job->covered_once && !job->aux.st && !job->greedy_all && !job->rade_all &&
+      (uint64_t)job->members * (uint64_t)job->nw <= kAsideWords) {
+    job->covered_once = true;
+    mcera_enqueue(job, k, job->st, h + gb, true);
+    greedy_enqueue(job, k, job->st, h, true);
+    CEN_CK(cudaStreamSynchronize(job->st));
+    if (!greedy_result(h, S, S_size, covered)) greedy_over_all(job, k, h, S, S_size, covered);
+    if (!mcera_result(job, k, h + gb, Rnum, Wnum, b)) mcera_over_all(job, k, h + gb, Rnum, Wnum, b);
+    return;
+  }
   job->aux.ensure();
   CEN_CK(cudaEventRecord(job->aux.fork, job->st));
   CEN_CK(cudaStreamWaitEvent(job->aux.st, job->aux.fork, 0));

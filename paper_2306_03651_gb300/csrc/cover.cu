@@ -92,12 +92,13 @@ void build_incidence(cen_job *job) {
   Stats *S = &job->stats;
   const int32_t n = job->g->n;
   const size_t members = (size_t)job->members;
-  job->c.ensure(4 * (size_t)n, st);
+  job->c.ensure(heavy_ctl_at(job) + sizeof(HeavyCtl), st);
   job->noff.ensure(8 * ((size_t)n + 1), st);
   job->nsamp.ensure(4 * (members + 1), st);
   job->hmemh.ensure(4 * (members + 1), st);
   job->heavy_m = ~0ull;
-  CEN_CK(cudaMemsetAsync(job->c.p, 0, 4 * (size_t)n, st));
+  CEN_CK(cudaMemsetAsync(job->c.p, 0, heavy_ctl_at(job) + sizeof(HeavyCtl), st));
+  job->heavy_clear = true;
   if (members)
     launch(S, K_TRANSPOSE, st, [&] {
       const bool wide = members >= kRankWide;
@@ -235,13 +236,13 @@ void build_heavy(cen_job *job) {
   const int32_t n = job->g->n;
   const bool all = n <= kHeavyMax;
   const size_t most = all ? (size_t)n : (size_t)kHeavyMax;
-  job->hctl.ensure(sizeof(HeavyCtl), st);
   job->hlist.ensure(4 * most, st);
   job->hc.ensure(4 * most, st);
   job->hidx.ensure(all ? 4 : 4 * (size_t)n, st);
   job->hchunks.ensure(8 * heavy_chunks_most(job, most), st);
-  HeavyCtl *ctl = job->hctl.as<HeavyCtl>();
-  CEN_CK(cudaMemsetAsync(ctl, 0, all ? offsetof(HeavyCtl, hist) : sizeof(HeavyCtl), st));
+  HeavyCtl *ctl = heavy_ctl(job);
+  if (!job->heavy_clear) CEN_CK(cudaMemsetAsync(ctl, 0, sizeof(HeavyCtl), st));  // (a call that failed left it)
+  job->heavy_clear = false;
   if (!all)
     launch(S, K_TRANSPOSE, st, [&] {
       k_heavy_hist<<<grid_for((size_t)n, 256 * 8, sm_count() * 4), 256, 0, st>>>(job->c.as<int32_t>(), n, ctl);
@@ -262,7 +263,7 @@ void build_heavy(cen_job *job) {
 }
 
 HeavyView heavy_view(const cen_job *job) {
-  return HeavyView{job->hctl.as<HeavyCtl>(), job->hlist.as<int32_t>(), job->hc.as<int32_t>(),
+  return HeavyView{heavy_ctl(job), job->hlist.as<int32_t>(), job->hc.as<int32_t>(),
                    job->hchunks.as<uint2>()};
 }
 
@@ -541,6 +542,12 @@ constexpr int64_t kGreedyClusterMaxPer = (227 * 1024 - 2048) / 4;
 
 size_t greedy_result_bytes(int32_t k) { return sizeof(GreedyCtl) + 4 * (size_t)k; }
 
+// The covered bits lie behind the control words and are cleared with them.
+static size_t greedy_control_bytes(int32_t k) { return (greedy_result_bytes(k) + 15) & ~(size_t)15; }
+static uint32_t *greedy_covered(const cen_job *job, int32_t k) {
+  return (uint32_t *)(job->gctl.as<char>() + greedy_control_bytes(k));
+}
+
 // Whether a cluster of C CTAs of `kernel` with `smem` bytes can be resident on
 // this device (the kernel's shared-memory limit is raised, and clusters over 8
 // allowed, once per device).
@@ -609,7 +616,7 @@ static bool greedy_cluster(cen_job *job, int32_t k, int64_t items, cudaStream_t 
       CEN_CK(cudaLaunchKernelEx(&cfg, k_greedy_cluster<HEAVY>, (const int32_t *)job->c.as<int32_t>(), heavy_view(job),
                                 (const int64_t *)job->noff.as<int64_t>(), (const int32_t *)job->nsamp.as<int32_t>(),
                                 (const int64_t *)job->hoff.as<int64_t>(), members, job->g->n,
-                                job->covered.as<uint32_t>(), ctl, (int)k, lg));
+                                greedy_covered(job, k), ctl, (int)k, lg));
     });
     return true;
   }
@@ -622,8 +629,7 @@ void greedy_prepare(cen_job *job, int32_t k) {
   CEN_REQUIRE(k >= 1, CEN_EINVAL, "cen_greedy_cover: k must be >= 1");
   cudaStream_t st = job->st;
   job->gain.ensure(4 * (size_t)job->g->n, st);
-  job->covered.ensure(4 * ((job->m + 31) / 32 + 1), st);
-  job->gctl.ensure(greedy_result_bytes(k), st);
+  job->gctl.ensure(greedy_control_bytes(k) + 4 * ((job->m + 31) / 32 + 1), st);
 }
 
 // Enqueues greedyCover(k) on stream `run` (after greedy_prepare), over the
@@ -633,8 +639,8 @@ void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool 
   Stats *St = &job->stats;
   const int32_t n = job->g->n;
   const size_t cbytes = greedy_result_bytes(k);
-  CEN_CK(cudaMemsetAsync(job->covered.p, 0, 4 * ((job->m + 31) / 32 + 1), run));
-  CEN_CK(cudaMemsetAsync(job->gctl.p, 0, cbytes, run));
+  CEN_CK(cudaMemsetAsync(job->gctl.p, 0, greedy_control_bytes(k) + 4 * ((job->m + 31) / 32 + 1), run));
+  uint32_t *const cov = greedy_covered(job, k);
   GreedyCtl *ctl = job->gctl.as<GreedyCtl>();
   // diagnostic: CEN_GREEDY_GRID=1 keeps the cooperative grid form
   const char *grid_env = getenv("CEN_GREEDY_GRID");
@@ -655,7 +661,7 @@ void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool 
     const int32_t *a_hmem = job->hmem.as<int32_t>();
     int32_t *a_gain = job->gain.as<int32_t>();
     int32_t a_n = n;
-    uint32_t *a_cov = job->covered.as<uint32_t>();
+    uint32_t *a_cov = cov;
     int a_k = k;
     void *args[] = {&a_noff, &a_nsamp, &a_hoff, &a_hmem, &a_gain, &a_n, &a_cov, &ctl, &a_k};
     launch(St, K_GREEDY, run, [&] {
@@ -670,7 +676,7 @@ void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool 
       launch(St, K_GREEDY, run, [&] {
         k_greedy_update<<<sm_count() * 4, 256, 0, run>>>(job->noff.as<int64_t>(), job->nsamp.as<int32_t>(),
                                                    job->hoff.as<int64_t>(), job->hmem.as<int32_t>(),
-                                                   job->gain.as<int32_t>(), job->covered.as<uint32_t>(), ctl, slot,
+                                                   job->gain.as<int32_t>(), cov, ctl, slot,
                                                    it);
       });
     }

@@ -48,6 +48,9 @@ struct HeavyView {
   const uint2 *chunks;      // (list entry, chunk of its row)
 };
 
+// Its control words lie behind the counts c and are cleared with them.
+inline size_t heavy_ctl_at(const cen_job *job) { return (4 * (size_t)job->g->n + 15) & ~(size_t)15; }
+inline HeavyCtl *heavy_ctl(const cen_job *job) { return (HeavyCtl *)(job->c.as<char>() + heavy_ctl_at(job)); }
 HeavyView heavy_view(const cen_job *job);
 // The list of all n nodes (entry u = node u) and the chunks of their rows; ctl's head is zero.
 void heavy_list_all(const int32_t *c, int32_t n, HeavyCtl *ctl, int32_t *list, int32_t *hc, uint2 *chunks,

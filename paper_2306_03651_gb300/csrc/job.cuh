@@ -135,8 +135,9 @@ struct cen_job {
   cen::DevBuf c, noff, nsamp;
   uint64_t inc_m = ~0ull;
   // heavy nodes of the sample (heavy.cuh) and whether the last greedy / AMCERA needed all nodes
-  cen::DevBuf hctl, hlist, hc, hidx, hchunks, hmemh;
+  cen::DevBuf hlist, hc, hidx, hchunks, hmemh;
   uint64_t heavy_m = ~0ull;
+  bool heavy_clear = false;  // the list's control words are zero
   bool greedy_all = false, rade_all = false;
   // greedy workspace
   cen::DevBuf gain, covered, gctl;
@@ -147,6 +148,7 @@ struct cen_job {
   int32_t rade_valid_k = -1;
   // greedyCover and AMCERA side by side (cen_cover_and_mcera)
   cen::AuxStream aux;
+  bool covered_once = false;  // such a call has run
   // sampler pipelines (workspace 0 runs on the job's stream)
   std::vector<std::unique_ptr<cen::WaveWS>> wws;
   int wave_streams = 4;  // waves of one cen_sample call run at once
