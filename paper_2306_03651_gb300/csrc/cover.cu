@@ -739,6 +739,7 @@ void shard_greedy_begin(cen_job *job) {
   greedy_prepare(job, 1);
   cudaStream_t st = job->st;
   const int32_t n = job->g->n;
+  job->covered.ensure(4 * ((job->m + 31) / 32 + 1), st);
   CEN_CK(cudaMemsetAsync(job->covered.p, 0, 4 * ((job->m + 31) / 32 + 1), st));
   launch(&job->stats, K_GREEDY, st,
          [&] { k_gain_init<<<grid_for(n, 256), 256, 0, st>>>(job->c.as<int32_t>(), job->gain.as<int32_t>(), n); });

@@ -139,8 +139,8 @@ struct cen_job {
   uint64_t heavy_m = ~0ull;
   bool heavy_clear = false;  // the list's control words are zero
   bool greedy_all = false, rade_all = false;
-  // greedy workspace
-  cen::DevBuf gain, covered, gctl;
+  // greedy workspace: gains, control words and covered bits; covered bits of a shard's picks
+  cen::DevBuf gain, gctl, covered;
   // AMCERA workspace
   cen::DevBuf R, selh, selst;
   cen::DevBuf Rh, hchunks_all, hctl_all, hlist_all, hc_all;  // over the heavy nodes; the chunks of all rows
