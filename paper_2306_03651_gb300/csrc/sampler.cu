@@ -1374,7 +1374,11 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   bidir_setup(job, m_new);
   BiWS &bw = *job->bws;
   const double mean = job->m ? (double)job->members / (double)job->m : 4.0;
+  // Twice the mean so far and, as a job's first samples have none, at least 64 a sample up to
+  // 64 MB: an arena that turns out short has the samples searched twice (65,536 pairs of the
+  // 2048^2 rewired grid, 36 members each: 194 ms a round, and 97 with this).
   int64_t cap = (int64_t)((double)m_new * std::max(8.0, 2.0 * mean)) + ((int64_t)1 << 20);
+  cap = std::max(cap, std::min<int64_t>((int64_t)m_new * 64, (int64_t)1 << 24));
   bw.arena.ensure(4 * (size_t)cap, st);
   int stages = 0;
   BiCtl h = bidir_search(job, m0, m_new, cap, &stages);
