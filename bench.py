@@ -153,7 +153,7 @@ class ClockSampler:
 
 
 # kernel class -> (committed ncu summary, source file whose hash it records)
-DRAM_PROFILES = {"expand_pull": ("expand_pull_dram.md", "sampler.cu"), "bidir": ("bidir_dram.md", "bidir.cu")}
+DRAM_PROFILES = {"expand_pull": ("expand_pull_dram.md", "sampler.cu"), "bidir": ("bidir_dram.md", "bidir_log.cuh")}
 
 
 def dram_traffic(kernel_class: str, workload: str, pairs_per_step: int):
@@ -394,8 +394,8 @@ def run_gpu(args, rank, world):
                 "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs)" if peak_src == "measured" else peak_src,
                 "avg_launch_ms": avg_ms, "launches": stats[dom]["launches"],
                 "algorithmic_bytes_per_launch": per_launch_bytes,
-                "note": ("one launch samples the whole step; the kernel is bound by the latency of dependent L2 "
-                         f"accesses ({ratio})"
+                "note": ("the step's searches in one to four launches, each for what the one before hands on; bound by "
+                         f"instruction issue and the latency of short dependent phases ({ratio})"
                          if dom == "bidir" else
                          "per-launch event times of concurrent wave pipelines include sharing the GPU"),
                 "aggregate_counted_GBps": counted / (total_ms / 1e3) / 1e9}

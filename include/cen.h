@@ -138,10 +138,13 @@ int cen_sample(cen_job *job, uint64_t m_new);
 /* Alg. 1 "greedyCover(k, H)" (Sec. 3.1): k times add the node covering the
  * most still-uncovered samples (lowest id on ties); stop early when that
  * count is 0.  S_out[k] (host) receives the picks in order, *S_size their
- * number, *covered = |{j : h_j meets S}| = m * C_H(S).  Runs as one
- * thread-block cluster holding the gains in shared memory when they fit (16
- * CTAs, n <= 921,600, where the device allows such clusters; else 8 CTAs,
- * n <= 460,800), otherwise as one cooperative grid launch.  Diagnostics (the
+ * number, *covered = |{j : h_j meets S}| = m * C_H(S).  Goes over
+ * the (at most 16,384) nodes in the most samples, in one thread-block cluster
+ * holding their gains in shared memory (16 CTAs where the device allows such
+ * clusters, else 8); when a pick's gain falls below what another node may have,
+ * it is repeated over all nodes, and the job's later calls go over all nodes at
+ * once: by such a cluster when the gains fit (n <= 921,600, or 460,800 by 8
+ * CTAs), otherwise as one cooperative grid launch.  Diagnostics (the
  * picks are the same): the environment variable CEN_GREEDY_CLUSTER=8 keeps
  * 8-CTA clusters, CEN_GREEDY_GRID=1 the grid form. */
 int cen_greedy_cover(cen_job *job, int32_t k, int32_t *S_out, int32_t *S_size, uint64_t *covered);
@@ -156,7 +159,8 @@ int cen_mcera(cen_job *job, int32_t k, int64_t *Rnum_out, int64_t *Wnum_out, int
 /* cen_greedy_cover and cen_mcera of one Alg. 1 round in one call, with the same
  * outputs: the two read the same sample and write disjoint buffers, so the
  * greedy runs on the job's stream while the AMCERA runs on a second stream
- * of the job (made on first use).  Synchronous at return; host outputs as
+ * of the job (made on first use; a job's first call of little work runs both on
+ * the job's stream).  Synchronous at return; host outputs as
  * above.  cen_run uses it for every CentRA round. */
 int cen_cover_and_mcera(cen_job *job, int32_t k, int32_t *S_out, int32_t *S_size, uint64_t *covered,
                         int64_t *Rnum_out, int64_t *Wnum_out, int32_t *b_out);
@@ -339,7 +343,9 @@ int cen_job_copy_samples(const cen_job *job, int64_t *hoff, int32_t *hmem, int32
  * nsamp[members] (each node's sample ids, as a set: order within a row is
  * unspecified).  Either may be NULL. */
 int cen_job_copy_incidence(const cen_job *job, int64_t *noff, int32_t *nsamp);
-/* R[q * n + u] (int32, t x n) and c[n] from the last cen_mcera call. */
+/* R[q * n + u] (int32, t x n) and c[n] of the sample that the last cen_mcera
+ * call read.  cen_mcera itself needs R of the heavy nodes only: this call
+ * computes the rest (R may be NULL). */
 int cen_job_copy_rade(const cen_job *job, int32_t *R, int32_t *c);
 /* Packed sign words of samples [0, m): words[j * ceil(t/32) + w], bit q%32 of word q/32 set iff sigma_{q,j} = +1. */
 int cen_job_copy_signs(const cen_job *job, uint32_t *words);
