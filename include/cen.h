@@ -344,8 +344,12 @@ int cen_job_copy_samples(const cen_job *job, int64_t *hoff, int32_t *hmem, int32
  * unspecified).  Either may be NULL. */
 int cen_job_copy_incidence(const cen_job *job, int64_t *noff, int32_t *nsamp);
 /* R[q * n + u] (int32, t x n) and c[n] of the sample that the last cen_mcera
- * call read.  cen_mcera itself needs R of the heavy nodes only: this call
- * computes the rest (R may be NULL). */
+ * (or cen_cover_and_mcera) call read, also when the job has grown since (its
+ * incidence must then be current: a greedy or mcera call after the last
+ * cen_sample, else CEN_EINVAL).  Either may be NULL.  Where the AMCERA needed
+ * R of the heavy nodes only, this call sums the rest from the samples, in a
+ * buffer of its own (rows of n entries up to 256 MB in all, at least one, and
+ * one for c; CEN_ENOMEM when there is no room); the job is only read. */
 int cen_job_copy_rade(const cen_job *job, int32_t *R, int32_t *c);
 /* Packed sign words of samples [0, m): words[j * ceil(t/32) + w], bit q%32 of word q/32 set iff sigma_{q,j} = +1. */
 int cen_job_copy_signs(const cen_job *job, uint32_t *words);

@@ -404,11 +404,58 @@ void rade_all(cen_job *job, cudaStream_t run) {
   job->rade_all_m = job->m;
 }
 
-// R over all nodes for cen_job_copy_rade, when the AMCERA did not need it.
-void rade_for_copy(cen_job *job) {
-  if (job->rade_all_m == job->m) return;
-  rade_all_prepare(job);
-  rade_all(job, job->st);
+// Rows q0 .. q0 + rows - 1 of R (zero before) and, where c is not null, c of samples 0 .. m - 1: a warp per
+// sample, its lanes the rows.  For cen_job_copy_rade alone, bound by its atomics.
+__global__ void __launch_bounds__(256) k_rade_of_prefix(const int64_t *__restrict__ hoff,
+                                                        const int32_t *__restrict__ hmem, uint64_t m, int32_t n,
+                                                        int q0, int rows, int nw, const uint32_t *__restrict__ sign,
+                                                        int32_t *R, int32_t *c) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t nwarps = (uint64_t)gridDim.x * 8;
+  for (uint64_t j = (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5); j < m; j += nwarps) {
+    const uint32_t *row = sign + (int64_t)j * nw;
+    for (int64_t e = hoff[j]; e < hoff[j + 1]; ++e) {
+      const int32_t u = hmem[e];
+      for (int r = lane; r < rows; r += 32)
+        atomicAdd(&R[(int64_t)r * n + u], (row[(q0 + r) >> 5] >> ((q0 + r) & 31)) & 1u ? 1 : -1);
+      if (c && lane == 0) atomicAdd(&c[u], 1);
+    }
+  }
+}
+
+// R and c of the sample that the last AMCERA read (rade_m: the first samples of the store, which may have
+// grown), to the host.  Where job->R does not hold them they are summed from the store, as many rows at a
+// time as kRadeCopyBytes hold, in buffers of the call's own: the job is only read.
+constexpr size_t kRadeCopyBytes = (size_t)256 << 20;
+void rade_copy(const cen_job *job, int32_t *R, int32_t *c) {
+  cudaStream_t st = job->st;
+  const size_t n = (size_t)job->g->n;
+  const int t = job->t;
+  if (job->rade_all_m == job->rade_m) {
+    if (R) CEN_CK(cudaMemcpyAsync(R, job->R.p, 4 * n * t, cudaMemcpyDeviceToHost, st));
+    if (c) CEN_CK(cudaMemcpyAsync(c, job->R.as<int32_t>() + n * t, 4 * n, cudaMemcpyDeviceToHost, st));
+    CEN_CK(cudaStreamSynchronize(st));
+    return;
+  }
+  if (!R && !c) return;
+  const int most = R ? (int)std::max<size_t>(1, std::min<size_t>(t, kRadeCopyBytes / (4 * n))) : 0;
+  DevBuf buf;
+  buf.ensure_exact(4 * n * (most + 1), st);
+  int32_t *dc = buf.as<int32_t>() + n * most;
+  for (int q0 = 0; q0 < (R ? t : 1); q0 += std::max(1, most)) {
+    const int rows = std::min(most, t - q0);
+    CEN_CK(cudaMemsetAsync(buf.p, 0, 4 * n * (most + 1), st));
+    if (job->rade_m) {
+      k_rade_of_prefix<<<grid_for(job->rade_m, 8), 256, 0, st>>>(job->hoff.as<int64_t>(), job->hmem.as<int32_t>(),
+                                                                 job->rade_m, job->g->n, q0, rows, job->nw,
+                                                                 job->sign.as<uint32_t>(), buf.as<int32_t>(),
+                                                                 c && q0 == 0 ? dc : nullptr);
+      CEN_CK(cudaGetLastError());
+    }
+    if (rows) CEN_CK(cudaMemcpyAsync(R + n * q0, buf.p, 4 * n * rows, cudaMemcpyDeviceToHost, st));
+    if (c && q0 == 0) CEN_CK(cudaMemcpyAsync(c, dc, 4 * n, cudaMemcpyDeviceToHost, st));
+  }
+  CEN_CK(cudaStreamSynchronize(st));
 }
 
 // Sizes the AMCERA workspace (allocations ordered on the job's stream).  The
@@ -463,6 +510,7 @@ bool mcera_result(cen_job *job, int32_t k, const void *h, int64_t *Rnum, int64_t
   memcpy(&hb, hrows + t + 1, 4);
   *b = job->m ? hb : 0;
   job->rade_valid_k = k;
+  job->rade_m = job->m;
   return true;
 }
 

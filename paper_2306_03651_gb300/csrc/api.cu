@@ -578,11 +578,7 @@ int cen_job_copy_rade(const cen_job *job, int32_t *R, int32_t *c) {
   CEN_API_BEGIN
   CEN_REQUIRE(job && job->rade_valid_k >= 0 && job->inc_m == job->m, CEN_EINVAL,
               "cen_job_copy_rade: call cen_mcera first");
-  cudaStream_t st = job->st;
-  if (R) cen::rade_for_copy(const_cast<cen_job *>(job));
-  if (R) CEN_CK(cudaMemcpyAsync(R, job->R.p, 4 * (size_t)job->g->n * job->t, cudaMemcpyDeviceToHost, st));
-  if (c) CEN_CK(cudaMemcpyAsync(c, job->c.p, 4 * (size_t)job->g->n, cudaMemcpyDeviceToHost, st));
-  CEN_CK(cudaStreamSynchronize(st));
+  cen::rade_copy(job, R, c);
   CEN_API_END
 }
 

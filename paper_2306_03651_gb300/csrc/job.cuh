@@ -145,6 +145,7 @@ struct cen_job {
   cen::DevBuf R, selh, selst;
   cen::DevBuf Rh, hchunks_all, hctl_all, hlist_all, hc_all;  // over the heavy nodes; the chunks of all rows
   uint64_t rade_all_m = ~0ull;      // sample size that R holds every node's row of
+  uint64_t rade_m = 0;              // sample size that the last AMCERA read
   int32_t rade_valid_k = -1;
   // greedyCover and AMCERA side by side (cen_cover_and_mcera)
   cen::AuxStream aux;
@@ -216,7 +217,7 @@ void build_heavy(cen_job *job);
 void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool heavy);
 bool greedy_result(const void *h, int32_t *S, int32_t *S_size, uint64_t *covered);
 void greedy_over_all(cen_job *job, int32_t k, void *h, int32_t *S, int32_t *S_size, uint64_t *covered);
-void rade_for_copy(cen_job *job);
+void rade_copy(const cen_job *job, int32_t *R, int32_t *c);
 size_t mcera_result_bytes(const cen_job *job);
 void mcera_prepare(cen_job *job, int32_t k);
 void mcera_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool heavy);
