@@ -1395,10 +1395,10 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   // warp searches pay off when few outgrow a warp; each one handed on is searched twice
   const unsigned long long nbig = bw.WQ ? h.nout[0] : 0;
   // a size of search that handed on most of many samples is left out from now on (not when a
-  // short queue made it)
-  if (bw.tier != kTierGlobal && job->bidir_queue >= kBidirQueue) {
+  // short queue made it, nor behind warp searches, which leave it only the largest)
+  if (bw.tier != kTierGlobal && !bw.WQ && job->bidir_queue >= kBidirQueue) {
     int tier = bw.tier;
-    for (int k = bw.WQ ? 1 : 0; tier < kTierGlobal && k < stages; ++k, ++tier) {
+    for (int k = 0; tier < kTierGlobal && k < stages; ++k, ++tier) {
       const unsigned long long in = k ? h.nout[k - 1] : m_new;
       if (in < 512 || 2 * h.nout[k] <= in) break;
     }

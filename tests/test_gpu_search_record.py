@@ -1,0 +1,26 @@
+"""What calls record on a graph about the sizes of bidirectional search: which launches a later call makes.
+A call that starts with the small shared-memory CTAs makes two (small, wide) or four (and two for the
+few left), one that starts with the wide ones one or three, one with the tables in global memory one."""
+import pytest
+
+from paper_2306_03651_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+P = pytest.importorskip("paper_2306_03651_gb300")
+
+
+def launches(graph, m, seed=1, **params):
+    job = P.Job(graph, seed, 1)
+    job.tune(**params)
+    job.sample(m)
+    return job.stats()["bidir"]["launches"]
+
+
+def test_warp_searches_leave_no_record_for_cta_searches():
+    """On this grid some 43% of all searches outgrow the small CTAs, but more than half of those that the
+    warps hand on do; a later job without warp searches still starts small."""
+    g = I.grid_rewired(120, 120, 0.01, 1)
+    fresh, after = P.Graph.of(g), P.Graph.of(g)
+    launches(after, 3000, bidir_warps=1)
+    assert launches(fresh, 3000) == 2
+    assert launches(after, 3000) == 2
