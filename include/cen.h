@@ -375,18 +375,21 @@ int cen_job_copy_signs(const cen_job *job, uint32_t *words);
                                     2^10 .. 2^24 (at most H / 2) or 0 for none (searches use the large
                                     table of H entries only); either way every search uses the tables
                                     in global memory.  -1 (default): searches start in shared memory
-                                    where they can, and the small tables of those that cannot are
-                                    sized to about 80 MiB in all so that they stay in L2; a search
-                                    that fills half of its small table moves to the large one.  With
-                                    -1, once a call of 1,024 or more samples sees most searches move,
-                                    later jobs on the graph use no small table */
+                                    where they can; those that outgrow it use the large table only.
+                                    On graphs of more than 2^24 nodes, where none can, the small
+                                    tables are sized to about 80 MiB in all so that they stay in L2,
+                                    a search that fills half of its small table moves to the large
+                                    one, and once a call of 1,024 or more samples sees most searches
+                                    move, later jobs on the graph use no small table */
 #define CEN_PARAM_BIDIR_WARPS 9  /* 1: each warp of a CTA searches samples alone with a 1,024-entry
                                     node table, and a second launch searches with whole CTAs those it
                                     hands on (a level of more than 2,048 arcs to expand, more than 512
                                     nodes, or more than 64 levels a side); 0: every sample is searched
-                                    by a whole CTA; -1 (default): 0 while the CTAs' searches start in
-                                    shared memory and on graphs whose degrees have E[d^2]/E[d] > 256
-                                    (frontiers that soon outgrow a warp), else 1 until a call of 1,024
+                                    by a whole CTA; -1 (default): 0 where the CTAs' searches can start
+                                    in shared memory (table size -1, at most 2^24 nodes), once calls on
+                                    the graph have seen most searches outgrow the smallest of those
+                                    CTAs, and on graphs whose degrees have E[d^2]/E[d] > 256
+                                    (frontiers that soon outgrow a warp); else 1 until a call of 1,024
                                     or more samples hands more than 30% on, then 0 for later jobs on
                                     the graph.  Queues of fewer than 1,024
                                     nodes use CTA searches only */
@@ -400,7 +403,9 @@ int cen_release_cached(void);
 /* How the job's samples were drawn so far: samples the bidirectional search
  * left whole to the bit-parallel sampler (*deferred_search), samples whose walk
  * it left to it (*deferred_walk), searches that outgrew the small node table
- * or the shared memory of a wide CTA (*migrated), the CTAs (slots) the
+ * or, in shared memory, the wide CTA that took them up (*migrated: each once; once
+ * most do, the rest of a call goes to the larger searches untried and uncounted),
+ * the CTAs (slots) the
  * bidirectional search may have global workspace for (0 before its first use;
  * it is allocated when a search needs it), and
  * the warp searches handed on to whole CTAs because a level, the node count or

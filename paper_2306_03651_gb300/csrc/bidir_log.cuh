@@ -47,6 +47,7 @@ template <int T_, int H_, int NQ_, int LQ_, int ARCS_, int CTAS_>
 struct LogCfg {
   static constexpr int T = T_, H = H_, NQ = NQ_, LQ = LQ_, ARCS = ARCS_, CTAS = CTAS_;
   static constexpr int LV = 32;  // levels per side
+  static constexpr bool WIDE = T_ == 512;  // the size whose hand-ons cen_job_sampler_info reports
   static constexpr int U = T_ > 128 ? 4 : 1;  // arcs of a lane per turn of the filtered scan
   static constexpr int FLOG = T_ > 256 ? 17 : T_ > 128 ? 16 : 15, FW = 1 << (FLOG - 5);  // bits and words of the frontier filter
   static_assert(4 * FW + 14 * T_ <= 4 * H_, "the filter and the rows share the counts' memory");
@@ -174,11 +175,10 @@ __device__ __forceinline__ uint32_t log_pick(LogSh<C> &S, int n, uint32_t r, int
   }
 }
 
-// Searches sample jr; returns false when it is handed on.  `full` reports that
-// the table, queue or log was too small.  S.tab is zero.  Called by
-// the whole CTA.
+// Searches sample jr; returns false when it is handed on.  S.tab is zero.
+// Called by the whole CTA.
 template <class C>
-__device__ __forceinline__ bool log_search(const BiArgs &A, LogSh<C> &S, uint64_t jr, int QC, bool &full) {
+__device__ __forceinline__ bool log_search(const BiArgs &A, LogSh<C> &S, uint64_t jr, int QC) {
   constexpr int T = C::T, H = C::H;
   const int tid = threadIdx.x, lane = tid & 31;
   const uint64_t j = A.j0 + jr;
@@ -228,7 +228,6 @@ __device__ __forceinline__ bool log_search(const BiArgs &A, LogSh<C> &S, uint64_
     x = c0 < c1 || (c0 == c1 && S.lvl[0] <= S.lvl[1]) ? 0 : 1;
     L = S.lvl[x];
     const uint32_t fcost = x ? c1 : c0;
-    full = false;
     if (L + 1 >= C::LV || fcost > (uint32_t)C::ARCS) return false;
     const int f0 = S.lo[x][L], f1 = S.lo[x][L + 1], base = S.nodes;
     const int64_t *__restrict__ o = x ? A.roff : A.off;
@@ -450,10 +449,7 @@ __device__ __forceinline__ bool log_search(const BiArgs &A, LogSh<C> &S, uint64_
       S.seg[x][L] = S.logged;
       S.sege[x][L] = S.logged = S.nlog;
     }
-    if (stop & ~1) {  // without the whole log, or a level cut short
-      full = true;
-      if (stop != 3) return false;
-    }
+    if ((stop & ~1) && stop != 3) return false;  // without the whole log, or a level cut short
     if (stop & 1) break;
     if (nadd == 0) break;  // this side's ball is closed: t is unreachable
     // arcs out of the new level
@@ -477,7 +473,6 @@ __device__ __forceinline__ bool log_search(const BiArgs &A, LogSh<C> &S, uint64_
     }
     __syncthreads();
   }
-  full = false;
   const bool met = S.stop & 1;  // (else t is unreachable)
   const int ls = S.lvl[0], lb = S.lvl[1];
   const int d = met ? ls + lb + 1 : -1;
@@ -675,13 +670,11 @@ __global__ void __launch_bounds__(C::T, C::CTAS) k_bidir_log(BiArgs A) {
       S.item[par ^ 1] = nx;
       S.skip[par ^ 1] = out > 256 && 2 * out > nx;
     }
-    bool full = false;
     __syncthreads();
-    if (skip || !log_search<C>(A, S, jr, QC, full)) {
+    if (skip || !log_search<C>(A, S, jr, QC)) {
       if (tid == 0) {
         A.out[atomicAdd(A.out_count, 1ull)] = jr;
-        if ((LIST || C::T > 128) && (full || (skip && 2 * ld_vol(&A.ctl->nmigrate) > ld_vol(A.out_count))))
-          atomicAdd(&A.ctl->nmigrate, 1ull);
+        if (C::WIDE && !skip) atomicAdd(&A.ctl->noutgrown, 1ull);
       }
     } else if (tid == 0) {
       arcs += S.arcs;

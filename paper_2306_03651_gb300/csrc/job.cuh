@@ -61,7 +61,8 @@ struct BiCtl {
   unsigned long long cursor;   // arena entries reserved
   unsigned long long nsearch;  // samples left whole to the bit-parallel sampler
   unsigned long long nwalk;    // samples whose walk is left to it (distance known)
-  unsigned long long nmigrate; // searches that outgrew the small table
+  unsigned long long nmigrate; // searches that outgrew the small table in global memory
+  unsigned long long noutgrown; // searches that wide CTAs took up and handed on
   int err;
   int pad;
 };

@@ -1294,10 +1294,13 @@ void bidir_setup(cen_job *job, uint64_t m_new) {
   while (H2 < 4 * QC) H2 *= 2;
   // searches start in shared memory unless a table size was set or the ids are too long for it
   const int tier = job->bidir_table < 0 && bidir_shared_ok(n) ? job->g->bidir_tier.load() : kTierGlobal;
-  // by default, warp searches only where that does not hold and frontiers grow slowly (E[d^2] / E[d],
-  // the mean degree at the far end of an arc, at most kWarpBranching), and until a call hands too many on
+  // By default, warp searches and small tables only where no record says that searches outgrow the
+  // small CTAs (they outgrow a warp and a small table then too); warps only where frontiers grow slowly
+  // (E[d^2] / E[d], the mean degree at the far end of an arc, at most kWarpBranching), and until a
+  // call hands too many on.
+  const bool unknown = tier == kTierGlobal && job->g->bidir_tier.load() == kTierSmall;
   const bool warps = job->bidir_warps > 0 ||
-                     (job->bidir_warps < 0 && tier == kTierGlobal && !job->g->bidir_warps_off.load() &&
+                     (job->bidir_warps < 0 && unknown && !job->g->bidir_warps_off.load() &&
                       graph_branching(job->g, st) <= kWarpBranching);
   const int64_t WQ = warps ? bidir_warp_queue(QC) : 0;
   auto per_slot = [&](int64_t h1) {
@@ -1306,7 +1309,7 @@ void bidir_setup(cen_job *job, uint64_t m_new) {
   const size_t res = (size_t)bidir_resident_slots();
   int slots = (int)std::min<size_t>(res, std::max<size_t>(1, job->bidir_budget / per_slot(0)));
   int64_t H1 = 0;
-  if (job->bidir_table < 0 && tier == kTierGlobal && !job->g->bidir_table_off.load()) {
+  if (job->bidir_table < 0 && unknown && !job->g->bidir_table_off.load()) {
     H1 = 1024;
     while ((size_t)(2 * H1) * 8 * (size_t)slots <= kTableL2 && 2 * H1 < H2) H1 *= 2;
   } else if (job->bidir_table > 0) {
@@ -1391,7 +1394,7 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
     bw.arena.ensure(4 * (size_t)cap, st);
     h = bidir_search(job, m0, m_new, cap, &stages);
   }
-  if (job->bidir_table < 0 && m_new >= 1024 && 2 * h.nmigrate > m_new) job->g->bidir_table_off.store(true);
+  if (job->bidir_table < 0 && bw.H1 && m_new >= 1024 && 2 * h.nmigrate > m_new) job->g->bidir_table_off.store(true);
   // warp searches pay off when few outgrow a warp; each one handed on is searched twice
   const unsigned long long nbig = bw.WQ ? h.nout[0] : 0;
   // a size of search that handed on most of many samples is left out from now on (not when a
@@ -1403,7 +1406,6 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
       if (in < 512 || 2 * h.nout[k] <= in) break;
     }
     if (tier > bw.tier) job->g->bidir_tier.store(tier);
-    if (tier == kTierGlobal) job->g->bidir_warps_off.store(true);  // such searches outgrow a warp too
   }
   if (job->bidir_warps < 0 && bw.WQ && m_new >= 1024 && 10 * nbig > 3 * m_new) job->g->bidir_warps_off.store(true);
   std::vector<uint64_t> search(h.nsearch), walk(h.nwalk);
@@ -1457,7 +1459,7 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   rerun_in_place(job, walk);
   job->bidir_deferred_search += h.nsearch;
   job->bidir_deferred_walk += walk.size();
-  job->bidir_migrated += h.nmigrate;
+  job->bidir_migrated += h.nmigrate + h.noutgrown;
   job->bidir_escalated += nbig;
   return total;
 }

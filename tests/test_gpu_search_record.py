@@ -24,3 +24,10 @@ def test_warp_searches_leave_no_record_for_cta_searches():
     launches(after, 3000, bidir_warps=1)
     assert launches(fresh, 3000) == 2
     assert launches(after, 3000) == 2
+
+
+def test_searches_that_outgrow_a_wide_cta_are_counted_once():
+    """Nearly all of these outgrow the wide CTAs, and most of those the 1,024-thread ones too."""
+    job = P.Job(P.Graph.of(I.grid_rewired(2048, 2048, 0.01, 1)), 1, 1)
+    job.sample(400)
+    assert job.stats()["bidir"]["launches"] == 4 and 200 < job.sampler_info()["migrated"] <= 400
