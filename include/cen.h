@@ -403,8 +403,7 @@ int cen_release_cached(void);
 /* How the job's samples were drawn so far: samples the bidirectional search
  * left whole to the bit-parallel sampler (*deferred_search), samples whose walk
  * it left to it (*deferred_walk), searches that outgrew the small node table
- * or, in shared memory, the wide CTA that took them up (*migrated: each once; once
- * most do, the rest of a call goes to the larger searches untried and uncounted),
+ * or, in shared memory, were left by the wide CTAs to larger ones (*migrated),
  * the CTAs (slots) the
  * bidirectional search may have global workspace for (0 before its first use;
  * it is allocated when a search needs it), and

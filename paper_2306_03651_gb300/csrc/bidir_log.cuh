@@ -47,7 +47,7 @@ template <int T_, int H_, int NQ_, int LQ_, int ARCS_, int CTAS_>
 struct LogCfg {
   static constexpr int T = T_, H = H_, NQ = NQ_, LQ = LQ_, ARCS = ARCS_, CTAS = CTAS_;
   static constexpr int LV = 32;  // levels per side
-  static constexpr bool WIDE = T_ == 512;  // the size whose hand-ons cen_job_sampler_info reports
+  static constexpr bool WIDE = T_ == 512;
   static constexpr int U = T_ > 128 ? 4 : 1;  // arcs of a lane per turn of the filtered scan
   static constexpr int FLOG = T_ > 256 ? 17 : T_ > 128 ? 16 : 15, FW = 1 << (FLOG - 5);  // bits and words of the frontier filter
   static_assert(4 * FW + 14 * T_ <= 4 * H_, "the filter and the rows share the counts' memory");
@@ -83,7 +83,7 @@ struct LogSh {
   int stop;                     // 1: the balls touched, 2: table or queue full, 4: log full
   int ovf;                      // a path count wrapped
   uint32_t ps, pt;              // table positions of s and t
-  uint32_t item[2], skip[2];
+  uint32_t item[2], skip[2], none;
   uint32_t red[C::T / 32];
   unsigned long long arcs;
 };
@@ -644,7 +644,14 @@ __device__ __forceinline__ bool log_search(const BiArgs &A, LogSh<C> &S, uint64_
 }
 
 // Searches of every sample of the launch, or (LIST) of the listed ones.  Once
-// most of what was taken has been handed on, the rest follows unsearched.
+// most of what was taken has been handed on, the rest follows unsearched.  In the
+// wide CTAs it also does where most searches are deep and some were handed on: a
+// graph's first call, of which many are left to search, finds out here that they
+// are better off in global memory (see kManyDeep), or before it takes up any when
+// the small CTAs could finish hardly one.  The fewer are handed on, the more must be left
+// (first rounds on 1% rewired grids, searched here to the end and not, ms: 500 a side, 10%
+// handed on, 3,000 pairs 3.45 and 3.84, 4,500 4.77 and 3.91; 350, 1%, 4,500 pairs 2.96 and
+// 3.38, 8,000 4.78 and 4.17).
 template <class C, bool LIST>
 __global__ void __launch_bounds__(C::T, C::CTAS) k_bidir_log(BiArgs A) {
   extern __shared__ uint4 smem4[];
@@ -655,7 +662,10 @@ __global__ void __launch_bounds__(C::T, C::CTAS) k_bidir_log(BiArgs A) {
   unsigned long long arcs = 0;
   if (tid == 0) {
     S.item[0] = (uint32_t)atomicAdd(A.next, 1ull);
-    S.skip[0] = 0;
+    // whether to take up none: many, of which the small CTAs finished one in sixteen at most, those not shallow
+    S.none = C::WIDE && LIST && count > kManyLeft * 3 / 2 && 16 * (A.count - count) < count &&
+             ld_vol(&A.ctl->cursor) > 8 * (A.count - count);
+    S.skip[0] = S.none;
   }
   for (int par = 0;; par ^= 1) {
     __syncthreads();
@@ -663,21 +673,27 @@ __global__ void __launch_bounds__(C::T, C::CTAS) k_bidir_log(BiArgs A) {
     if (i >= count) break;
     const uint32_t skip = S.skip[par];
     const uint64_t jr = LIST ? A.list[i] : i;
-    for (int p = tid; p < C::H / 4; p += C::T) ((uint4 *)S.tab)[p] = make_uint4(0, 0, 0, 0);
+    if (!skip)
+      for (int p = tid; p < C::H / 4; p += C::T) ((uint4 *)S.tab)[p] = make_uint4(0, 0, 0, 0);
     if (tid == C::T - 32) {  // the next item, fetched while this one is set up
       const uint32_t nx = (uint32_t)atomicAdd(A.next, 1ull);
       const unsigned long long out = ld_vol(A.out_count);
+      bool rest = (out > 256 && 2 * out > nx) || (C::WIDE && S.none);
+      if (C::WIDE && out && nx + kManyLeft < count) {
+        const unsigned long long deep = out + ld_vol(&A.ctl->ndeep), left = count - nx;
+        rest |= deep > 256 && 2 * deep > nx && (left > 4096 || left * out > 256ull * nx);
+      }
       S.item[par ^ 1] = nx;
-      S.skip[par ^ 1] = out > 256 && 2 * out > nx;
+      S.skip[par ^ 1] = rest;
     }
     __syncthreads();
     if (skip || !log_search<C>(A, S, jr, QC)) {
       if (tid == 0) {
         A.out[atomicAdd(A.out_count, 1ull)] = jr;
-        if (C::WIDE && !skip) atomicAdd(&A.ctl->noutgrown, 1ull);
       }
     } else if (tid == 0) {
       arcs += S.arcs;
+      if (C::WIDE && S.lvl[0] + S.lvl[1] >= (int)kDeepLevels) atomicAdd(&A.ctl->ndeep, 1ull);
     }
   }
   if (tid == 0 && arcs) atomicAdd(A.units, arcs * 4ull);  // an arc read; its lookup stays in shared memory

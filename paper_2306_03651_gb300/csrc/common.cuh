@@ -328,9 +328,12 @@ struct cen_graph {
   // Set once most bidirectional searches on this graph outgrew their node
   // table: later jobs (without an explicit table size) use the large table only.
   mutable std::atomic<bool> bidir_table_off{false};
-  // Where CTA searches on this graph start (kTier*): raised once a call handed
-  // most of its searches on.
-  mutable std::atomic<int> bidir_tier{0};
+  // Samples that the small CTAs of shared-memory searches have seen, how many of
+  // them they handed on, and whether that was most (the wide CTAs come first then).
+  mutable std::atomic<uint64_t> bidir_seen{0}, bidir_handed{0};
+  mutable std::atomic<bool> bidir_wide{false};
+  // Samples of a call from which such searches start with the tables in global memory.
+  mutable std::atomic<uint64_t> bidir_many{~0ull};
   // Set once a call handed more than 30% of its warp searches on to CTAs:
   // later jobs (without an explicit setting) search with whole CTAs only.
   mutable std::atomic<bool> bidir_warps_off{false};

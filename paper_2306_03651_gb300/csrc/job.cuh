@@ -62,7 +62,7 @@ struct BiCtl {
   unsigned long long nsearch;  // samples left whole to the bit-parallel sampler
   unsigned long long nwalk;    // samples whose walk is left to it (distance known)
   unsigned long long nmigrate; // searches that outgrew the small table in global memory
-  unsigned long long noutgrown; // searches that wide CTAs took up and handed on
+  unsigned long long ndeep;    // deep searches (kDeepLevels) that the wide CTAs finished
   int err;
   int pad;
 };
@@ -71,6 +71,17 @@ struct BiCtl {
 // memory, or the tables in global memory.
 constexpr int64_t kBidirQueue = (int64_t)1 << 16;  // default queue entries per ball or cone side
 constexpr int kTierSmall = 0, kTierWide = 1, kTierGlobal = 2;
+// Where most searches outgrow the small CTAs, a call of few samples starts wide and one of many with the tables in
+// global memory, where eight times as many searches are in flight: a deep search waits at each of its levels, most
+// of them small, so that many at once hide more than fast memory saves.  Rounds on 1% rewired grids (18 to 34 arcs
+// between a pair), wide against global, ms: 200 x 200 (the wide CTAs leave nothing) 2,000 pairs 1.14 and 1.10, 2,500
+// 1.31 and 1.19, 8,000 3.14 and 2.50; 500 x 500 (10% left) 1,000 pairs 1.57 and 2.21, 1,500 2.42 and 1.83, 8,000 6.65
+// and 4.05; 1,400 x 1,400 (78% left) 700 pairs 3.78 and 4.01, 900 4.65 and 4.20, and 2,000 x 2,000 800 pairs 5.77 and
+// 6.39, 1,000 6.98 and 7.15.  Shallow searches (R-MAT, BA) stay in shared memory however many they are.
+constexpr uint64_t kDeepLevels = 12;  // levels of both balls, or arcs between a pair less one, of a deep search
+constexpr uint64_t kManyDeep = 2048;  // many, where the wide CTAs leave nothing,
+constexpr uint64_t kManyLeft = 1024;  // some,
+constexpr uint64_t kManyMost = 896;   // three in four
 struct BiWS {
   DevBuf tab1, tab2, lists, sig, epochs, ctl, aoff, dsearch, dwalk, arena;
   DevBuf tabw, epw;        // warp searches: node tables and epochs (none when WQ = 0)

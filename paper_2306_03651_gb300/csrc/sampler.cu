@@ -1292,13 +1292,18 @@ void bidir_setup(cen_job *job, uint64_t m_new) {
   const int64_t QC = std::max<int64_t>(16, std::min<int64_t>(n, job->bidir_queue));
   int64_t H2 = 1024;
   while (H2 < 4 * QC) H2 *= 2;
-  // searches start in shared memory unless a table size was set or the ids are too long for it
-  const int tier = job->bidir_table < 0 && bidir_shared_ok(n) ? job->g->bidir_tier.load() : kTierGlobal;
+  // searches start in shared memory unless a table size was set, the ids are too long for it, or the call has
+  // many of those that would not stay there
+  const bool wide = job->g->bidir_wide.load();
+  const int tier = job->bidir_table >= 0 || !bidir_shared_ok(n)     ? kTierGlobal
+                   : !wide                                          ? kTierSmall
+                   : m_new < job->g->bidir_many.load()              ? kTierWide
+                                                                    : kTierGlobal;
   // By default, warp searches and small tables only where no record says that searches outgrow the
   // small CTAs (they outgrow a warp and a small table then too); warps only where frontiers grow slowly
   // (E[d^2] / E[d], the mean degree at the far end of an arc, at most kWarpBranching), and until a
   // call hands too many on.
-  const bool unknown = tier == kTierGlobal && job->g->bidir_tier.load() == kTierSmall;
+  const bool unknown = tier == kTierGlobal && !wide;
   const bool warps = job->bidir_warps > 0 ||
                      (job->bidir_warps < 0 && unknown && !job->g->bidir_warps_off.load() &&
                       graph_branching(job->g, st) <= kWarpBranching);
@@ -1369,6 +1374,27 @@ static BiCtl bidir_search(cen_job *job, uint64_t m0, uint64_t m_new, int64_t cap
   return bidir_finish(job);
 }
 
+// What a call's shared-memory searches show of the graph: whether most outgrow the small CTAs (over all calls, so
+// that short ones settle too), and then from how many samples on a call starts in global memory.
+static void bidir_record(const cen_graph *g, int tier, uint64_t m_new, const BiCtl &h) {
+  if (tier == kTierSmall) {
+    const uint64_t handed = g->bidir_handed += h.nout[0], seen = g->bidir_seen += m_new;
+    if (seen >= 512 && 2 * handed > seen) g->bidir_wide.store(true);
+  }
+  if (!g->bidir_wide.load()) return;
+  const uint64_t in = tier == kTierSmall ? h.nout[0] : m_new, left = h.nout[tier == kTierSmall ? 1 : 0];
+  const bool deep = h.cursor >= kDeepLevels * m_new;
+  uint64_t many = ~0ull;
+  if (in >= 512 && 4 * left > 3 * in)
+    many = kManyMost;
+  else if (left && (deep || (in >= 512 && 2 * left > in)))
+    many = kManyLeft;
+  else if (deep)
+    many = kManyDeep;
+  for (uint64_t was = g->bidir_many.load(); many < was && !g->bidir_many.compare_exchange_weak(was, many);) {
+  }
+}
+
 // Bidirectional form: one CTA per sample writes its members to an arena;
 // what it defers runs on the bit-parallel sampler (see bidir.cu).  Returns
 // the new members.
@@ -1397,16 +1423,9 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   if (job->bidir_table < 0 && bw.H1 && m_new >= 1024 && 2 * h.nmigrate > m_new) job->g->bidir_table_off.store(true);
   // warp searches pay off when few outgrow a warp; each one handed on is searched twice
   const unsigned long long nbig = bw.WQ ? h.nout[0] : 0;
-  // a size of search that handed on most of many samples is left out from now on (not when a
-  // short queue made it, nor behind warp searches, which leave it only the largest)
-  if (bw.tier != kTierGlobal && !bw.WQ && job->bidir_queue >= kBidirQueue) {
-    int tier = bw.tier;
-    for (int k = 0; tier < kTierGlobal && k < stages; ++k, ++tier) {
-      const unsigned long long in = k ? h.nout[k - 1] : m_new;
-      if (in < 512 || 2 * h.nout[k] <= in) break;
-    }
-    if (tier > bw.tier) job->g->bidir_tier.store(tier);
-  }
+  // learnt from calls whose CTA searches see every sample and have queues of full length
+  if (bw.tier != kTierGlobal && !bw.WQ && job->bidir_queue >= kBidirQueue)
+    bidir_record(job->g, bw.tier, m_new, h);
   if (job->bidir_warps < 0 && bw.WQ && m_new >= 1024 && 10 * nbig > 3 * m_new) job->g->bidir_warps_off.store(true);
   std::vector<uint64_t> search(h.nsearch), walk(h.nwalk);
   if (h.nsearch)
@@ -1459,7 +1478,8 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   rerun_in_place(job, walk);
   job->bidir_deferred_search += h.nsearch;
   job->bidir_deferred_walk += walk.size();
-  job->bidir_migrated += h.nmigrate + h.noutgrown;
+  job->bidir_migrated += h.nmigrate;
+  if (bw.tier != kTierGlobal) job->bidir_migrated += h.nout[(bw.WQ ? 1 : 0) + (bw.tier == kTierSmall ? 1 : 0)];
   job->bidir_escalated += nbig;
   return total;
 }

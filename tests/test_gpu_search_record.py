@@ -31,3 +31,16 @@ def test_searches_that_outgrow_a_wide_cta_are_counted_once():
     job = P.Job(P.Graph.of(I.grid_rewired(2048, 2048, 0.01, 1)), 1, 1)
     job.sample(400)
     assert job.stats()["bidir"]["launches"] == 4 and 200 < job.sampler_info()["migrated"] <= 400
+
+
+def test_short_calls_settle_on_the_wide_ctas():
+    """Most of this grid's searches outgrow the small CTAs and none the wide ones: calls of 300 learn it together."""
+    graph = P.Graph.of(I.grid_rewired(200, 200, 0.01, 1))
+    assert [launches(graph, 300, seed) for seed in range(4)] == [2, 2, 1, 1]
+
+
+def test_many_deep_searches_start_in_global_memory_and_few_do_not():
+    """Here the wide CTAs leave 10%.  The first call of 8,000 finds that out on the way (small, wide, and the rest
+    with the tables in global memory), later ones start there; a call of 500 stays in shared memory."""
+    graph = P.Graph.of(I.grid_rewired(500, 500, 0.01, 1))
+    assert [launches(graph, m, 1) for m in (8000, 8000, 500, 8000)] == [3, 1, 3, 1]
