@@ -142,9 +142,9 @@ int cen_sample(cen_job *job, uint64_t m_new);
  * the (at most 16,384) nodes in the most samples, in one thread-block cluster
  * holding their gains in shared memory (16 CTAs where the device allows such
  * clusters, else 8); when a pick's gain falls below what another node may have,
- * it is repeated over all nodes, and the job's later calls go over all nodes at
- * once: by such a cluster when the gains fit (n <= 921,600, or 460,800 by 8
- * CTAs), otherwise as one cooperative grid launch.  Diagnostics (the
+ * it goes on over all nodes (the job's later calls of as large a k at once, where
+ * that came before half of the picks): by such a cluster when the gains fit (n <=
+ * 921,600, or 460,800 by 8 CTAs), otherwise as one cooperative grid launch.  Diagnostics (the
  * picks are the same): the environment variable CEN_GREEDY_CLUSTER=8 keeps
  * 8-CTA clusters, CEN_GREEDY_GRID=1 the grid form. */
 int cen_greedy_cover(cen_job *job, int32_t k, int32_t *S_out, int32_t *S_size, uint64_t *covered);

@@ -465,7 +465,7 @@ void mcera_prepare(cen_job *job, int32_t k) {
   cudaStream_t st = job->st;
   const int nrows = job->t + 1;
   job->selst.ensure(sizeof(SelRow) * (size_t)nrows, st);
-  if (!job->rade_all) {
+  if (k < job->rade_all_k) {
     job->Rh.ensure(4 * (size_t)std::min(job->g->n, kHeavyMax) * job->t, st);
     return;
   }
@@ -516,7 +516,7 @@ bool mcera_result(cen_job *job, int32_t k, const void *h, int64_t *Rnum, int64_t
 
 // The AMCERA over all nodes, on the job's stream.
 static void mcera_over_all(cen_job *job, int32_t k, void *h, int64_t *Rnum, int64_t *Wnum, int32_t *b) {
-  job->rade_all = true;  // the job's later samples spread over as many nodes
+  job->rade_all_k = std::min(job->rade_all_k, k);
   mcera_prepare(job, k);
   mcera_enqueue(job, k, job->st, h, false);
   CEN_CK(cudaStreamSynchronize(job->st));
@@ -544,7 +544,7 @@ void cover_and_mcera(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint6
   mcera_prepare(job, k);
   const size_t gb = (greedy_result_bytes(k) + 15) & ~(size_t)15;
   char *h = (char *)host_staging(job, gb + mcera_result_bytes(job));
-  if (!job->covered_once && !job->aux.st && !job->greedy_all && !job->rade_all &&
+  if (!job->covered_once && !job->aux.st && k < job->greedy_all_k && k < job->rade_all_k &&
       (uint64_t)job->members * (uint64_t)job->nw <= kAsideWords) {
     job->covered_once = true;
     mcera_enqueue(job, k, job->st, h + gb, true);
@@ -557,9 +557,9 @@ void cover_and_mcera(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint6
   job->aux.ensure();
   CEN_CK(cudaEventRecord(job->aux.fork, job->st));
   CEN_CK(cudaStreamWaitEvent(job->aux.st, job->aux.fork, 0));
-  greedy_enqueue(job, k, job->st, h, !job->greedy_all);
+  greedy_enqueue(job, k, job->st, h, k < job->greedy_all_k);
   try {
-    mcera_enqueue(job, k, job->aux.st, h + gb, !job->rade_all);
+    mcera_enqueue(job, k, job->aux.st, h + gb, k < job->rade_all_k);
   } catch (...) {  // still join, so that nothing on the job's stream outruns the second stream
     cudaEventRecord(job->aux.join, job->aux.st);
     cudaStreamWaitEvent(job->st, job->aux.join, 0);
@@ -610,7 +610,7 @@ void mcera(cen_job *job, int32_t k, int64_t *Rnum, int64_t *Wnum, int32_t *b) {
   build_heavy(job);
   mcera_prepare(job, k);
   void *h = host_staging(job, mcera_result_bytes(job));
-  mcera_enqueue(job, k, job->st, h, !job->rade_all);
+  mcera_enqueue(job, k, job->st, h, k < job->rade_all_k);
   CEN_CK(cudaStreamSynchronize(job->st));
   if (!mcera_result(job, k, h, Rnum, Wnum, b)) mcera_over_all(job, k, h, Rnum, Wnum, b);
 }

@@ -282,6 +282,19 @@ __global__ void k_gain_init(const int32_t *__restrict__ c, int32_t *gain, int32_
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) gain[i] = c[i];
 }
 
+// Lowers the gains of the members of the covered samples, GS lanes a sample.
+template <int GS>
+__global__ void __launch_bounds__(256) k_gain_drop(const int64_t *__restrict__ hoff, const int32_t *__restrict__ hmem,
+                                                   uint64_t m, const uint32_t *__restrict__ covered, int32_t *gain) {
+  const int lane = threadIdx.x & (GS - 1);
+  const uint64_t groups = (uint64_t)gridDim.x * 256 / GS;
+  for (uint64_t j = ((uint64_t)blockIdx.x * 256 + threadIdx.x) / GS; j < m; j += groups) {
+    if (!((covered[j >> 5] >> (j & 31)) & 1u)) continue;
+    const int64_t e1 = hoff[j + 1];
+    for (int64_t e = hoff[j] + lane; e < e1; e += GS) atomicSub(&gain[hmem[e]], 1);
+  }
+}
+
 // argmax over nodes of key = gain << 32 | (2^32 - 1 - u): the max key has the
 // largest gain and, among equal gains, the lowest id.
 __global__ void __launch_bounds__(256) k_greedy_argmax(const int32_t *__restrict__ gain, int32_t n, GreedyCtl *ctl,
@@ -340,7 +353,8 @@ __global__ void __launch_bounds__(256) k_greedy_update(const int64_t *__restrict
 
 // All k iterations in one cooperative launch: each iteration is the argmax
 // (block maxima, one atomicMax per block), a grid barrier, the update of the
-// picked node's samples, and another barrier.  The picks, ties and counts
+// picked node's samples, and another barrier.  The first ctl->size picks are
+// made already.  The picks, ties and counts
 // are those of k_greedy_argmax / k_greedy_update.  A cooperative launch runs
 // only when every block is resident at once, so the barriers always complete.
 __global__ void __launch_bounds__(256) k_greedy_all(const int64_t *__restrict__ noff, const int32_t *__restrict__ nsamp,
@@ -351,7 +365,7 @@ __global__ void __launch_bounds__(256) k_greedy_all(const int64_t *__restrict__ 
   __shared__ unsigned long long wb[8];
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int it = 0; it < k; ++it) {
+  for (int it = ctl->size; it < k; ++it) {  // (size is first written behind a grid barrier)
     const int slot = it & 1;
     unsigned long long best = 0;
     for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
@@ -399,8 +413,9 @@ __global__ void __launch_bounds__(256) k_greedy_all(const int64_t *__restrict__ 
 // CTA reads the others' keys through distributed shared memory and so picks
 // the same u*; then a thread per incident sample of u* sets the sample's
 // covered bit and, if it was not set, decrements the gains of the sample's
-// members in their owners' shared memory; another cluster barrier.  The picks
-// and counts are those of k_greedy_all.  A cluster is launched only when all
+// members in their owners' shared memory; another cluster barrier.  With
+// HEAVY = false the first ctl->size picks are made already, and `gains` follow from
+// them.  The picks and counts are those of k_greedy_all.  A cluster is launched only when all
 // of its CTAs are resident at once, so the barriers always complete.
 //
 // Over the heavy nodes a CTA holds at most 1,024 gains (two keys a thread), so
@@ -416,7 +431,7 @@ constexpr int kGreedyThreads = 512;
 
 template <bool HEAVY>
 __global__ void __launch_bounds__(kGreedyThreads, 1)
-    k_greedy_cluster(const int32_t *__restrict__ c, HeavyView H, const int64_t *__restrict__ noff,
+    k_greedy_cluster(const int32_t *__restrict__ gains, HeavyView H, const int64_t *__restrict__ noff,
                      const int32_t *__restrict__ nsamp, const int64_t *__restrict__ hoff,
                      const int32_t *__restrict__ hmem, int32_t n, uint32_t *covered, GreedyCtl *ctl, int k, int lg) {
   extern __shared__ int64_t s_items[];
@@ -447,16 +462,17 @@ __global__ void __launch_bounds__(kGreedyThreads, 1)
       s_id[i] = u;
       s_row[i] = noff[u];
     } else {
-      s_gain[i] = c[i * C + rank];
+      s_gain[i] = gains[i * C + rank];
     }
   }
+  const int first = HEAVY ? 0 : ctl->size;
   cl.sync();
   // a sample's members are dealt to 2^lg lanes
   const int gl = tid & ((1 << lg) - 1);
   const unsigned gmask = (lg == 5 ? 0xffffffffu : (1u << (1 << lg)) - 1u) << (lane & ~((1 << lg) - 1));
   const int64_t gt = ((int64_t)rank * kGreedyThreads + tid) >> lg;
   const int64_t ngroups = ((int64_t)C * kGreedyThreads) >> lg;
-  for (int it = 0; it < k; ++it) {
+  for (int it = first; it < k; ++it) {
     uint32_t bg = 0, bi = 0;  // the thread's best gain, and the complement of its node
     int32_t bat = 0;
     for (int32_t i = tid; i < mine; i += kGreedyThreads) {
@@ -586,10 +602,11 @@ static bool greedy_cluster_ready(K kernel, int C, size_t smem) {
 }
 
 // Enqueues k_greedy_cluster<HEAVY> over `items` gains in the largest cluster
-// that holds them; false when none does.  Diagnostic: CEN_GREEDY_CLUSTER=8
+// that holds them (`gains` of all nodes when not HEAVY); false when none does.  Diagnostic: CEN_GREEDY_CLUSTER=8
 // keeps the portable cluster size.
 template <bool HEAVY>
-static bool greedy_cluster(cen_job *job, int32_t k, int64_t items, cudaStream_t run, GreedyCtl *ctl) {
+static bool greedy_cluster(cen_job *job, int32_t k, int64_t items, const int32_t *gains, cudaStream_t run,
+                           GreedyCtl *ctl) {
   const char *size_env = getenv("CEN_GREEDY_CLUSTER");
   // the members of a sample as list entries, and lanes for about its mean number of members
   const int32_t *members = (HEAVY && job->g->n > kHeavyMax ? job->hmemh : job->hmem).as<int32_t>();
@@ -613,7 +630,7 @@ static bool greedy_cluster(cen_job *job, int32_t k, int64_t items, cudaStream_t 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     launch(&job->stats, K_GREEDY, run, [&] {
-      CEN_CK(cudaLaunchKernelEx(&cfg, k_greedy_cluster<HEAVY>, (const int32_t *)job->c.as<int32_t>(), heavy_view(job),
+      CEN_CK(cudaLaunchKernelEx(&cfg, k_greedy_cluster<HEAVY>, gains, heavy_view(job),
                                 (const int64_t *)job->noff.as<int64_t>(), (const int32_t *)job->nsamp.as<int32_t>(),
                                 (const int64_t *)job->hoff.as<int64_t>(), members, job->g->n,
                                 greedy_covered(job, k), ctl, (int)k, lg));
@@ -634,32 +651,48 @@ void greedy_prepare(cen_job *job, int32_t k) {
 
 // Enqueues greedyCover(k) on stream `run` (after greedy_prepare), over the
 // heavy nodes or over all; the result reaches hdst (pinned,
-// greedy_result_bytes(k)) once `run` has drained.
-void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool heavy) {
+// greedy_result_bytes(k)) once `run` has drained.  With made > 0 (over all
+// nodes) the control words and covered bits hold that many picks already, and
+// their gains are taken from the covered bits.
+static void greedy_enqueue_from(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool heavy, int made) {
   Stats *St = &job->stats;
   const int32_t n = job->g->n;
   const size_t cbytes = greedy_result_bytes(k);
-  CEN_CK(cudaMemsetAsync(job->gctl.p, 0, greedy_control_bytes(k) + 4 * ((job->m + 31) / 32 + 1), run));
   uint32_t *const cov = greedy_covered(job, k);
   GreedyCtl *ctl = job->gctl.as<GreedyCtl>();
+  const int32_t *gains = job->c.as<int32_t>();
+  if (made) {
+    CEN_CK(cudaMemsetAsync(&ctl->short_, 0, sizeof(ctl->short_), run));
+    int32_t *left = job->gain_left.as<int32_t>();
+    launch(St, K_GREEDY, run, [&] { k_gain_init<<<grid_for(n, 256), 256, 0, run>>>(gains, left, n); });
+    launch(St, K_GREEDY, run, [&] {
+      const bool wide = job->members > kShortMembers * (int64_t)job->m;
+      auto kernel = wide ? k_gain_drop<32> : k_gain_drop<4>;
+      kernel<<<grid_for(job->m * (wide ? 32 : 4), 256), 256, 0, run>>>(job->hoff.as<int64_t>(),
+                                                                       job->hmem.as<int32_t>(), job->m, cov, left);
+    });
+    gains = left;
+  } else {
+    CEN_CK(cudaMemsetAsync(job->gctl.p, 0, greedy_control_bytes(k) + 4 * ((job->m + 31) / 32 + 1), run));
+  }
   // diagnostic: CEN_GREEDY_GRID=1 keeps the cooperative grid form
   const char *grid_env = getenv("CEN_GREEDY_GRID");
   const bool grid_form = grid_env && grid_env[0] == '1';
-  const bool done = !grid_form && (heavy ? greedy_cluster<true>(job, k, std::min<int64_t>(n, kHeavyMax), run, ctl)
-                                         : greedy_cluster<false>(job, k, n, run, ctl));
+  const bool done = !grid_form && (heavy ? greedy_cluster<true>(job, k, std::min<int64_t>(n, kHeavyMax), gains, run, ctl)
+                                         : greedy_cluster<false>(job, k, n, gains, run, ctl));
   if (done) {
     CEN_CK(cudaMemcpyAsync(hdst, ctl, cbytes, cudaMemcpyDeviceToHost, run));
     return;
   }
-  launch(St, K_GREEDY, run,
-         [&] { k_gain_init<<<grid_for(n, 256), 256, 0, run>>>(job->c.as<int32_t>(), job->gain.as<int32_t>(), n); });
+  int32_t *const work = made ? job->gain_left.as<int32_t>() : job->gain.as<int32_t>();
+  if (!made) launch(St, K_GREEDY, run, [&] { k_gain_init<<<grid_for(n, 256), 256, 0, run>>>(gains, work, n); });
   const int coop = cooperative_grid((const void *)k_greedy_all, 256);
   if (coop > 0) {
     const int64_t *a_noff = job->noff.as<int64_t>();
     const int32_t *a_nsamp = job->nsamp.as<int32_t>();
     const int64_t *a_hoff = job->hoff.as<int64_t>();
     const int32_t *a_hmem = job->hmem.as<int32_t>();
-    int32_t *a_gain = job->gain.as<int32_t>();
+    int32_t *a_gain = work;
     int32_t a_n = n;
     uint32_t *a_cov = cov;
     int a_k = k;
@@ -669,15 +702,13 @@ void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool 
     });
   } else {
     const int gblocks = grid_for((size_t)n, 256, sm_count() * 4);
-    for (int it = 0; it < k; ++it) {
+    for (int it = made; it < k; ++it) {
       const int slot = it & 1;
-      launch(St, K_GREEDY, run,
-             [&] { k_greedy_argmax<<<gblocks, 256, 0, run>>>(job->gain.as<int32_t>(), n, ctl, slot); });
+      launch(St, K_GREEDY, run, [&] { k_greedy_argmax<<<gblocks, 256, 0, run>>>(work, n, ctl, slot); });
       launch(St, K_GREEDY, run, [&] {
         k_greedy_update<<<sm_count() * 4, 256, 0, run>>>(job->noff.as<int64_t>(), job->nsamp.as<int32_t>(),
                                                    job->hoff.as<int64_t>(), job->hmem.as<int32_t>(),
-                                                   job->gain.as<int32_t>(), cov, ctl, slot,
-                                                   it);
+                                                   work, cov, ctl, slot, it);
       });
     }
   }
@@ -695,10 +726,21 @@ bool greedy_result(const void *h, int32_t *S, int32_t *S_size, uint64_t *covered
   return true;
 }
 
-// greedyCover over all nodes, on the job's stream (greedy_prepare done).
+void greedy_enqueue(cen_job *job, int32_t k, cudaStream_t run, void *hdst, bool heavy) {
+  greedy_enqueue_from(job, k, run, hdst, heavy, 0);
+}
+
+// Goes on over all nodes, on the job's stream, where the heavy ones left the
+// copied result h.  Their picks stand: each gain was at least tau, and no other
+// node's can be.  A call of as many picks or more goes over all nodes at once
+// where they were less than half.  A first round's greedy and AMCERA, the picks made
+// again, over all nodes alone, and as it is: ring of 60,000 nodes, 40,000 walks, k =
+// 6,000 28.5, 22.0, 19.9 ms; BA n = 200,000, 65,536 walks, k = 3,000 19.2, 11.9, 10.0.
 void greedy_over_all(cen_job *job, int32_t k, void *h, int32_t *S, int32_t *S_size, uint64_t *covered) {
-  job->greedy_all = true;  // the job's later samples spread over as many nodes
-  greedy_enqueue(job, k, job->st, h, false);
+  const int made = ((const GreedyCtl *)h)->size;
+  if (2 * (int64_t)made < k) job->greedy_all_k = std::min(job->greedy_all_k, k);
+  if (made) job->gain_left.ensure(4 * (size_t)job->g->n, job->st);
+  greedy_enqueue_from(job, k, job->st, h, false, made);
   CEN_CK(cudaStreamSynchronize(job->st));
   greedy_result(h, S, S_size, covered);
 }
@@ -800,7 +842,7 @@ void greedy_cover(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint64_t
   build_heavy(job);
   greedy_prepare(job, k);
   void *h = host_staging(job, greedy_result_bytes(k));
-  greedy_enqueue(job, k, job->st, h, !job->greedy_all);
+  greedy_enqueue(job, k, job->st, h, k < job->greedy_all_k);
   CEN_CK(cudaStreamSynchronize(job->st));
   if (!greedy_result(h, S, S_size, covered)) greedy_over_all(job, k, h, S, S_size, covered);
 }

@@ -8,8 +8,10 @@
 // raised a row's sum.  tau is the lowest bound of a c_u bucket that leaves at
 // most kHeavyMax nodes (1 when that many nodes or fewer are in a sample at
 // all).  Each use checks its condition on the device and reports when it does
-// not hold; the caller then repeats it over all nodes, and the job's later
-// calls go over all nodes at once.  Listing costs two passes over c_u (34 us
+// not hold; greedyCover then goes on over all nodes from the picks it has, the
+// AMCERA (some 50 us) is repeated over all.  A job's later calls of as large a k go
+// over all nodes at once (greedyCover: where less than half of the picks were made).
+// Listing costs two passes over c_u (34 us
 // for 4.2 million nodes).  Measured over all nodes against the heavy ones: a
 // round's greedy and AMCERA on directed R-MAT 22 (t = 100) 3.5 -> 0.4 ms, on the
 // rewired grid of 4.2 million nodes 4.4 -> 0.3 ms.

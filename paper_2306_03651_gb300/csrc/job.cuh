@@ -146,13 +146,13 @@ struct cen_job {
   // node -> sample incidence (rebuilt lazily when m changed)
   cen::DevBuf c, noff, nsamp;
   uint64_t inc_m = ~0ull;
-  // heavy nodes of the sample (heavy.cuh) and whether the last greedy / AMCERA needed all nodes
+  // heavy nodes of the sample (heavy.cuh) and the k from which greedyCover / the AMCERA go over all nodes at once
   cen::DevBuf hlist, hc, hidx, hchunks, hmemh;
   uint64_t heavy_m = ~0ull;
   bool heavy_clear = false;  // the list's control words are zero
-  bool greedy_all = false, rade_all = false;
-  // greedy workspace: gains, control words and covered bits; covered bits of a shard's picks
-  cen::DevBuf gain, gctl, covered;
+  int32_t greedy_all_k = INT32_MAX, rade_all_k = INT32_MAX;
+  // greedy workspace: gains, control words and covered bits; covered bits of a shard's picks; gains left by picks made
+  cen::DevBuf gain, gctl, covered, gain_left;
   // AMCERA workspace
   cen::DevBuf R, selh, selst;
   cen::DevBuf Rh, hchunks_all, hctl_all, hlist_all, hc_all;  // over the heavy nodes; the chunks of all rows
