@@ -68,12 +68,17 @@ def estimate_job_bytes(n: int, nnz: int, t: int, m_cap: int, avg_hyperedge: floa
     Bidirectional sampler: one workspace per resident CTA (a large node table
     and as many path counts, H = 4 `bidir_queue` entries each, seven lists of
     `bidir_queue` entries, and a small table of at most 80 MiB over all CTAs),
-    as many as fit in `bidir_budget`.  Wave workspace (the fallback): `levels` + 6 arrays
+    as many as fit in `bidir_budget`.  Searches in shared memory need none of it, but a call
+    that leaves many of them to global memory makes it all, and nothing tells beforehand:
+    it is counted in full.  Five lists of a call's samples and the member arena (at least 64
+    members a sample up to 64 MB, and 4 MB).  Wave workspace (the fallback): `levels` + 6 arrays
     of n*G words (G = wave words, at most 32 and at most 1 GB per array) and the
     initial cone-arc log (2 n G records of 24 bytes); sample store for m_cap
     samples: offsets, endpoints, distance, sign words and members (samples, incidence
-    and their places in it), plus the member arena; AMCERA table R[t+1][n] and greedy /
-    incidence arrays.  `resident_ctas` is the sampler's CTAs in flight (16 per SM
+    and their places in it), plus the arena's members; AMCERA table R[t+1][n], R[t] of
+    the heavy nodes, and the greedy and incidence arrays over all nodes (counts, offsets,
+    gains twice, list entries; the list of all nodes, their counts and the chunks of
+    their rows).  `resident_ctas` is the sampler's CTAs in flight (16 per SM
     on a 152-SM GB300)."""
     qc = max(16, min(n, bidir_queue))
     h2 = 1024
@@ -88,8 +93,9 @@ def estimate_job_bytes(n: int, nnz: int, t: int, m_cap: int, avg_hyperedge: floa
     wave = 8 * words * (levels + 6) + 24 * 2 * words
     nw = (t + 31) // 32
     store = m_cap * (8 + 12 + 4 * nw) + 4 * 4 * int(m_cap * avg_hyperedge)
-    node = n * (4 * (t + 1) + 4 * 4 + 8)
-    return int(bidir + wave + store + node)
+    lists = 5 * 8 * m_cap + 4 * (min(64 * m_cap, 1 << 24) + (1 << 20))
+    node = n * (4 * (t + 1) + 4 + 8 + 2 * 4 + 4 + 4 + 4 + 8) + 4 * t * min(n, 16384)
+    return int(bidir + wave + store + lists + node)
 
 
 def run_rounds(graph, req: Request, stream, reserve) -> dict:
