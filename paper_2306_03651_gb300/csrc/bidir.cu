@@ -1135,22 +1135,6 @@ __global__ void __launch_bounds__(kBiThreads, kBiWarpCtaPerSM) k_bidir_warp(BiAr
 
 #include "bidir_log.cuh"
 
-// The three sizes of shared-memory search.  Measured (R-MAT 18, 65,536 pairs,
-// against 5.33 ms with the tables in global memory): small 1.34 ms for all but
-// 3% of the searches, wide 0.42 ms for all of those.  The small one is bound by
-// instruction issue and the latency of short phases: 10 CTAs of 128 threads per
-// SM took 1.38 ms, 9 took 1.44 and 7 (with a table of 2,048 entries) 1.68;
-// 64-thread CTAs 1.57.  A level of more than 65,536 arcs goes to a wide CTA: at
-// 32,768 the small launch falls to 1.19 ms and the wide one rises to 0.61.
-// Nodes and logged arcs: the small one with 700 and 1,100 hands more on (the
-// batch's wide launches 2.3 -> 5.8 ms); the wide one with 5,600 and 8,192 left
-// a few R-MAT 18 searches to a huge one, 0.10 ms and a host synchronisation;
-// the huge one with 14,000 and 19,400 is slower on directed R-MAT 22 (0.25 ->
-// 0.38 ms), where one that does not fit either is searched longer in vain.
-using LogSmall = LogCfg<128, 1536, 1100, 1344, 65536, 10>;
-using LogWide = LogCfg<512, 7168, 6400, 10000, (1 << 24) - 1, 2>;
-using LogHuge = LogCfg<1024, 15360, 12288, 18432, (1 << 24) - 1, 1>;
-
 // ------------------------------------------------------------------ host
 int bidir_resident_slots() { return resident_grid((const void *)k_bidir<false>, kBiThreads); }
 
