@@ -54,21 +54,6 @@ __global__ void k_check_loops(const int64_t *__restrict__ off, const int32_t *__
   }
 }
 
-// The row that holds arc e of the offsets off[n + 1] (the last that starts at
-// or before it), by a whole warp: 32 probes a round.
-__device__ __forceinline__ int32_t warp_row(const int64_t *__restrict__ off, int32_t n, int64_t e) {
-  const int lane = threadIdx.x & 31;
-  int64_t lo = 0, hi = (int64_t)n + 1;
-  while (hi - lo > 1) {
-    const int64_t step = (hi - lo + 32) / 33, at = lo + (int64_t)(lane + 1) * step;
-    const int c = __popc(__ballot_sync(0xffffffffu, at < hi && off[at] <= e));
-    const int64_t nhi = lo + (int64_t)(c + 1) * step;
-    lo += (int64_t)c * step;
-    hi = nhi < hi ? nhi : hi;
-  }
-  return (int32_t)lo;
-}
-
 // Calls f(e, u) for every arc e with its row u.  A warp takes kArcRun
 // consecutive arcs, finds the rows of the first and the last, and each lane
 // searches its arcs' rows between them, so that work follows arcs and not
@@ -81,8 +66,8 @@ __device__ __forceinline__ void for_arcs(const int64_t *__restrict__ off, int32_
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t b = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kArcRun; b < nnz; b += nwarps * kArcRun) {
     const int64_t end = b + kArcRun < nnz ? b + kArcRun : nnz;
-    int32_t lo = warp_row(off, n, b);
-    const int32_t last = warp_row(off, n, end - 1);
+    int32_t lo = (int32_t)warp_upper(off, (int64_t)n + 1, b);  // the row of arc b: the last that starts at or before it
+    const int32_t last = (int32_t)warp_upper(off, (int64_t)n + 1, end - 1);
     for (int64_t e = b + lane; e < end; e += 32) {
       int32_t hi = last;  // off[lo] <= e
       while (lo < hi) {

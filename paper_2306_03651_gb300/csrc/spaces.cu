@@ -122,23 +122,6 @@ __global__ void __launch_bounds__(kWalkThreads) k_kpath(uint64_t j0, uint64_t co
   }
 }
 
-// The largest i in [0, count) with a[i] <= x (a ascending, a[0] <= x), by a
-// whole warp: 32 probes a round.
-__device__ __forceinline__ int64_t warp_upper(const int64_t *__restrict__ a, int64_t count, int64_t x) {
-  const int lane = threadIdx.x & 31;
-  int64_t lo = 0, hi = count;  // a[lo] <= x, and a[hi] > x or hi = count
-  while (hi - lo > 1) {
-    const int64_t step = (hi - lo + 32) / 33;
-    const int64_t at = lo + (int64_t)(lane + 1) * step;
-    const bool le = at < hi && a[at] <= x;
-    const int c = __popc(__ballot_sync(0xffffffffu, le));  // the probes ascend
-    const int64_t nhi = lo + (int64_t)(c + 1) * step;
-    lo += (int64_t)c * step;
-    hi = nhi < hi ? nhi : hi;
-  }
-  return lo;
-}
-
 // Common neighbours w > v of u and v, ascending: the shorter row's entries
 // above v, 128 at a time, are looked up in the longer row by binary search
 // (both rows are sorted, so either order of the two rows gives the same
