@@ -44,3 +44,11 @@ def test_many_deep_searches_start_in_global_memory_and_few_do_not():
     with the tables in global memory), later ones start there; a call of 500 stays in shared memory."""
     graph = P.Graph.of(I.grid_rewired(500, 500, 0.01, 1))
     assert [launches(graph, m, 1) for m in (8000, 8000, 500, 8000)] == [3, 1, 3, 1]
+
+
+def test_a_first_call_of_long_samples_is_searched_once():
+    """Some 21 members a sample, more than eight and the arena's spare million hold: a short arena would have the
+    samples searched twice."""
+    job = P.Job(P.Graph.of(I.grid_rewired(200, 200, 0.01, 1)), 1, 1)
+    job.sample(80000)
+    assert job.size()[1] > 8 * 80000 + (1 << 20) and job.stats()["bidir"]["launches"] == 2
