@@ -159,8 +159,8 @@ int cen_mcera(cen_job *job, int32_t k, int64_t *Rnum_out, int64_t *Wnum_out, int
 /* cen_greedy_cover and cen_mcera of one Alg. 1 round in one call, with the same
  * outputs: the two read the same sample and write disjoint buffers, so the
  * greedy runs on the job's stream while the AMCERA runs on a second stream
- * of the job (made on first use; a job's first call of little work runs both on
- * the job's stream).  Synchronous at return; host outputs as
+ * of the job (made on first use; a job's first call of very little work runs both
+ * on the job's stream).  Synchronous at return; host outputs as
  * above.  cen_run uses it for every CentRA round. */
 int cen_cover_and_mcera(cen_job *job, int32_t k, int32_t *S_out, int32_t *S_size, uint64_t *covered,
                         int64_t *Rnum_out, int64_t *Wnum_out, int32_t *b_out);

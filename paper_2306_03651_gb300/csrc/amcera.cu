@@ -523,13 +523,14 @@ static void mcera_over_all(cen_job *job, int32_t k, void *h, int64_t *Rnum, int6
   CEN_REQUIRE(mcera_result(job, k, h, Rnum, Wnum, b), CEN_ECUDA, "cen_mcera: the select left a row open");
 }
 
-// The first such call of a job that has at most this many sign words to read
-// (members x words) runs the AMCERA ahead of greedyCover on the job's stream:
-// its 10 us are less than the 20 a second stream takes to make and give back,
-// and many jobs make one call (BA 2,000, 50,000 members: a round's 222 us
-// instead of 235).  A job that calls again makes the second stream: without
-// it, the nine rounds of a certified run on that graph take 4.25 ms, not 4.11.
-constexpr uint64_t kAsideWords = (uint64_t)1 << 17;
+// The first such call of a job with at most this many nodes and sign words to
+// read (members x words) runs the AMCERA ahead of greedyCover on the job's stream:
+// there a second stream costs more to make and give back than it hides, and many
+// jobs make one call.  First call and release, one stream and two, us: BA n = 2,000,
+// 2,423 words 163 and 168, 9,692 161 and 165, 11,992 166 and 172, 28,771 180 and 172,
+// 120,130 213 and 192; R-MAT 14, 9,163 words 187 and 177; BA n = 200,000, 3,760 words 194
+// and 187.
+constexpr uint64_t kAsideWork = (uint64_t)1 << 14;
 
 // greedyCover on the job's stream and the AMCERA on its second stream at the
 // same time: the two read the same incidence and write disjoint buffers, so
@@ -545,7 +546,7 @@ void cover_and_mcera(cen_job *job, int32_t k, int32_t *S, int32_t *S_size, uint6
   const size_t gb = (greedy_result_bytes(k) + 15) & ~(size_t)15;
   char *h = (char *)host_staging(job, gb + mcera_result_bytes(job));
   if (!job->covered_once && !job->aux.st && k < job->greedy_all_k && k < job->rade_all_k &&
-      (uint64_t)job->members * (uint64_t)job->nw <= kAsideWords) {
+      (uint64_t)job->g->n + (uint64_t)job->members * (uint64_t)job->nw <= kAsideWork) {
     job->covered_once = true;
     mcera_enqueue(job, k, job->st, h + gb, true);
     greedy_enqueue(job, k, job->st, h, true);

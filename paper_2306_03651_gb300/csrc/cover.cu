@@ -418,7 +418,8 @@ __global__ void __launch_bounds__(256) k_greedy_all(const int64_t *__restrict__ 
 // them.  The picks and counts are those of k_greedy_all.  A cluster is launched only when all
 // of its CTAs are resident at once, so the barriers always complete.
 //
-// Over the heavy nodes a CTA holds at most 1,024 gains (two keys a thread), so
+// Over the heavy nodes a CTA of 16 holds at most 1,024 gains (two keys a thread;
+// of 8, 2,048), so
 // a pick costs its two barriers and the chain of loads of the picked row, some
 // 3.2 us: R-MAT 18, m = 65,536, k = 50: 0.21 -> 0.16 ms; directed R-MAT 22, k =
 // 100, whose 4.2 million gains no cluster holds: 3.2 -> 0.37 ms against the
