@@ -48,7 +48,7 @@ def test_many_deep_searches_start_in_global_memory_and_few_do_not():
 
 def test_a_first_call_of_long_samples_is_searched_once():
     """Some 21 members a sample, more than eight and the arena's spare million hold: a short arena would have the
-    samples searched twice."""
+    samples searched twice, in twice as many launches (small, wide, and in global memory the many that are left)."""
     job = P.Job(P.Graph.of(I.grid_rewired(200, 200, 0.01, 1)), 1, 1)
     job.sample(80000)
-    assert job.size()[1] > 8 * 80000 + (1 << 20) and job.stats()["bidir"]["launches"] == 2
+    assert job.size()[1] > 8 * 80000 + (1 << 20) and job.stats()["bidir"]["launches"] == 3
