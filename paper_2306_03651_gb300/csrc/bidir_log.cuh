@@ -706,6 +706,7 @@ __global__ void __launch_bounds__(C::T, C::CTAS) k_bidir_log(BiArgs A) {
     if (skip || !log_search<C>(A, S, jr, QC)) {
       if (tid == 0) {
         A.out[atomicAdd(A.out_count, 1ull)] = jr;
+        if (C::WIDE && !skip) atomicAdd(&A.ctl->noutgrown, 1ull);
       }
     } else if (tid == 0) {
       arcs += S.arcs;

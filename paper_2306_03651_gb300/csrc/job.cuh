@@ -63,6 +63,7 @@ struct BiCtl {
   unsigned long long nwalk;    // samples whose walk is left to it (distance known)
   unsigned long long nmigrate; // searches that outgrew the small table in global memory
   unsigned long long ndeep;    // deep searches (kDeepLevels) that the wide CTAs finished
+  unsigned long long noutgrown; // searches that they took up and handed on
   int err;
   int pad;
 };

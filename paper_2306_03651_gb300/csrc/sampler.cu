@@ -1383,11 +1383,12 @@ static void bidir_record(const cen_graph *g, int tier, uint64_t m_new, const BiC
   }
   if (!g->bidir_wide.load()) return;
   const uint64_t in = tier == kTierSmall ? h.nout[0] : m_new, left = h.nout[tier == kTierSmall ? 1 : 0];
+  const uint64_t tried = in - left + h.noutgrown;  // of which the wide CTAs handed noutgrown on
   const bool deep = h.cursor >= kDeepLevels * m_new;
   uint64_t many = ~0ull;
-  if (in >= 512 && 4 * left > 3 * in)
+  if (tried >= 256 && 4 * h.noutgrown > 3 * tried)
     many = kManyMost;
-  else if (left && (deep || (in >= 512 && 2 * left > in)))
+  else if (left && (deep || (tried >= 256 && 2 * h.noutgrown > tried)))
     many = kManyLeft;
   else if (deep)
     many = kManyDeep;

@@ -52,3 +52,9 @@ def test_a_first_call_of_long_samples_is_searched_once():
     job = P.Job(P.Graph.of(I.grid_rewired(200, 200, 0.01, 1)), 1, 1)
     job.sample(80000)
     assert job.size()[1] > 8 * 80000 + (1 << 20) and job.stats()["bidir"]["launches"] == 3
+
+
+def test_searches_left_untried_do_not_count_as_left_by_the_wide_ctas():
+    """The first call hands nearly all on untried; the wide CTAs would leave 10%, so a call of 950 still starts there."""
+    graph = P.Graph.of(I.grid_rewired(500, 500, 0.01, 1))
+    assert [launches(graph, m, 1) for m in (8000, 950)] == [3, 3]
