@@ -363,7 +363,9 @@ int cen_job_copy_signs(const cen_job *job, uint32_t *words);
                                     bit-parallel sampler for what exceeds its per-CTA limits (default);
                                     1: bit-parallel waves only.  Hyper-edges are identical.  On graphs of
                                     up to 2^24 nodes the searches keep their state in shared memory;
-                                    those that outgrow it use the global-memory workspace below. */
+                                    those that outgrow it, and once that is known of a graph the deep
+                                    searches of calls of many samples, use the global-memory workspace
+                                    below. */
 #define CEN_PARAM_BIDIR_BUDGET 6 /* device bytes for the bidirectional sampler's per-CTA workspace,
                                     >= 2^20 (default 2^34); fewer CTAs run when it is small.  One CTA
                                     needs 8 h + 16 H + 28 q bytes, plus 32,800 with warp searches

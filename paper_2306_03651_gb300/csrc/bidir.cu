@@ -23,8 +23,9 @@
 // and counts fit there, for graphs of up to 2^24 nodes.  What outgrows those
 // (deep searches such as a rewired grid's, or 2^32 paths) is searched with the
 // tables in global memory, as everything is on larger graphs or when a table
-// size is set.  A graph whose searches mostly outgrow a size skips it from the
-// next call on.  The rest of this comment describes the global-memory form.
+// size is set.  A graph whose searches mostly outgrow the small CTAs skips those
+// from then on, and where they are deep too, calls of many samples skip shared
+// memory (kManyDeep).  The rest of this comment describes the global-memory form.
 //
 // Two granularities run in two persistent launches of 128-thread CTAs.  In
 // the first, each warp takes sample ids from a counter and searches on its
