@@ -518,6 +518,8 @@ __device__ __forceinline__ bool row_has(const int32_t *__restrict__ c, int64_t e
 
 }  // namespace
 
+// In a list entry: the search had too many levels or paths for any size in shared memory.
+constexpr uint64_t kLongId = 1ull << 63;
 struct BiArgs {
   int32_t n;
   int64_t nnz;
@@ -1056,7 +1058,7 @@ __global__ void __launch_bounds__(kBiThreads, kBiCtaPerSM) k_bidir(BiArgs A) {
     __syncthreads();
     const unsigned long long i = s_item;
     if (i >= count) break;
-    bi_search<kBiThreads, kBiMaxLevels>(A, sh, cw, LIST ? A.list[i] : i);
+    bi_search<kBiThreads, kBiMaxLevels>(A, sh, cw, LIST ? A.list[i] & ~kLongId : i);
     if (tid == 0) s_arcs += sh.arcs;
   }
   if (tid == 0 && s_arcs) atomicAdd(A.units, s_arcs * 12ull);
@@ -1079,7 +1081,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_bidir_wide(BiArgs A) {
     __syncthreads();
     const unsigned long long i = s_item;
     if (i >= count) break;
-    bi_search<kWideThreads, kBiMaxLevels>(A, sh, cw, A.list[i]);
+    bi_search<kWideThreads, kBiMaxLevels>(A, sh, cw, A.list[i] & ~kLongId);
     if (tid == 0) s_arcs += sh.arcs;
   }
   if (tid == 0 && s_arcs) atomicAdd(A.units, s_arcs * 12ull);
@@ -1310,7 +1312,7 @@ void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, 
   BiWS &w = *job->bws;
   cudaStream_t st = job->st;
   CEN_CK(cudaMemsetAsync(w.ctl.p, 0, sizeof(BiCtl), st));
-  if (w.WQ || w.tier == kTierGlobal) bidir_tables(job, (uint64_t)w.nslots);
+  if (w.WQ || w.tier == kTierGlobal || w.straight) bidir_tables(job, (uint64_t)w.nslots);
   BiArgs a = bidir_args(job, j0, count, arena_cap);
   const int grid = (int)std::min<uint64_t>((uint64_t)w.nslots, count);
   int stage = 0;
@@ -1324,6 +1326,10 @@ void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, 
     case kTierSmall:
       log_launch<LogSmall>(job, a, count);
       next_stage(job, a, stage++);
+      if (w.straight) {
+        launch(&job->stats, K_BIDIR, st, [&] { k_bidir<true><<<grid, kBiThreads, 0, st>>>(a); });
+        break;
+      }
       [[fallthrough]];
     case kTierWide:
       log_launch<LogWide>(job, a, count);
@@ -1342,18 +1348,22 @@ void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, 
 // The `left` searches that bidir_launch's stages handed on.  A few (the last,
 // large ones of a call) go to CTAs of 1,024 threads, with their state in shared
 // memory if it fits and in global memory if not, so that they do not run on at
-// 128 threads each while the rest of the chip is idle; many go to the 128-thread
-// CTAs with the tables in global memory.
-void bidir_launch_rest(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages, uint64_t left) {
+// 128 threads each while the rest of the chip is idle; many, and those that are
+// long rather than large (not `wide`: most have too many levels or paths for shared
+// memory), go to the 128-thread CTAs with the tables in global memory, whose barriers
+// cost a level less (300 pairs of a cycle of 1,000 nodes 7.4 -> 3.8 ms).
+void bidir_launch_rest(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages, uint64_t left,
+                       bool wide) {
   BiWS &w = *job->bws;
   cudaStream_t st = job->st;
-  const int ctas = bidir_tables(job, left < kWideMost ? (uint64_t)sm_count() : (uint64_t)w.nslots);
+  wide &= left < kWideMost;
+  const int ctas = bidir_tables(job, wide ? (uint64_t)sm_count() : (uint64_t)w.nslots);
   const int grid = (int)std::min<uint64_t>((uint64_t)ctas, left);
   BiArgs a = bidir_args(job, j0, count, arena_cap);
   int stage = *stages;
   next_stage(job, a, stage - 1);
   next_stage(job, a, stage++);
-  if (left < kWideMost) {
+  if (wide) {
     log_launch<LogHuge>(job, a, left);
     next_stage(job, a, stage++);
     launch(&job->stats, K_BIDIR, st, [&] { k_bidir_wide<<<grid, kWideThreads, 0, st>>>(a); });

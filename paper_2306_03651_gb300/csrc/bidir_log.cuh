@@ -41,12 +41,12 @@ constexpr bool log_smooth(int h) {
   return h == 1;
 }
 
-// T threads; H table entries; NQ nodes (both balls); LQ logged arcs; a level
+// T threads; H table entries; NQ nodes (both balls); LQ logged arcs; LV levels per side; a level
 // of more than ARCS arcs is handed on; CTAS resident CTAs per SM.
-template <int T_, int H_, int NQ_, int LQ_, int ARCS_, int CTAS_>
+template <int T_, int H_, int NQ_, int LQ_, int LV_, int ARCS_, int CTAS_>
 struct LogCfg {
   static constexpr int T = T_, H = H_, NQ = NQ_, LQ = LQ_, ARCS = ARCS_, CTAS = CTAS_;
-  static constexpr int LV = 32;  // levels per side
+  static constexpr int LV = LV_;  // levels per side
   static constexpr bool WIDE = T_ == 512;
   static constexpr int U = T_ > 128 ? 4 : 1;  // arcs of a lane per turn of the filtered scan
   static constexpr int FLOG = T_ > 256 ? 17 : T_ > 128 ? 16 : 15, FW = 1 << (FLOG - 5);  // bits and words of the frontier filter
@@ -69,9 +69,13 @@ struct LogCfg {
 // a few R-MAT 18 searches to a huge one, 0.10 ms and a host synchronisation;
 // the huge one with 14,000 and 19,400 is slower on directed R-MAT 22 (0.25 ->
 // 0.38 ms), where one that does not fit either is searched longer in vain.
-using LogSmall = LogCfg<128, 1536, 1100, 1344, 65536, 10>;
-using LogWide = LogCfg<512, 7168, 6400, 10000, (1 << 24) - 1, 2>;
-using LogHuge = LogCfg<1024, 15360, 12288, 18432, (1 << 24) - 1, 1>;
+// Levels: as many as an entry's 6 bits and, in the small one, the memory of 10 CTAs
+// hold (with 60, 9 CTAs fit: R-MAT rounds 5% slower).  With 32 a cycle of 150 nodes,
+// whose searches have 38 levels of two nodes, took 3.9 ms a round of 3,000 pairs, all
+// but the levels' number fitting, against 1.24 in global memory; now 0.69.
+using LogSmall = LogCfg<128, 1536, 1100, 1344, 56, 65536, 10>;
+using LogWide = LogCfg<512, 7168, 6400, 10000, 62, (1 << 24) - 1, 2>;
+using LogHuge = LogCfg<1024, 15360, 12288, 18432, 62, (1 << 24) - 1, 1>;
 
 template <class C>
 struct LogSh {
@@ -664,7 +668,8 @@ __device__ __forceinline__ bool log_search(const BiArgs &A, LogSh<C> &S, uint64_
 // wide CTAs it also does where most searches are deep and some were handed on: a
 // graph's first call, of which many are left to search, finds out here that they
 // are better off in global memory (see kManyDeep), or before it takes up any when
-// the small CTAs could finish hardly one.  The fewer are handed on, the more must be left
+// the small CTAs could finish hardly one, or where most that it hands on have too
+// many levels or paths for any size (marked, for the huge CTAs to leave out).  The fewer are handed on, the more must be left
 // (first rounds on 1% rewired grids, searched here to the end and not, ms: 500 a side, 10%
 // handed on, 3,000 pairs 3.45 and 3.84, 4,500 4.77 and 3.91; 350, 1%, 4,500 pairs 2.96 and
 // 3.38, 8,000 4.78 and 4.17).
@@ -687,8 +692,9 @@ __global__ void __launch_bounds__(C::T, C::CTAS) k_bidir_log(BiArgs A) {
     __syncthreads();
     const uint32_t i = S.item[par];
     if (i >= count) break;
-    const uint32_t skip = S.skip[par];
+    uint32_t skip = S.skip[par];
     const uint64_t jr = LIST ? A.list[i] : i;
+    if constexpr (C::T > 512) skip |= jr >= kLongId;
     if (!skip)
       for (int p = tid; p < C::H / 4; p += C::T) ((uint4 *)S.tab)[p] = make_uint4(0, 0, 0, 0);
     if (tid == C::T - 32) {  // the next item, fetched while this one is set up
@@ -699,14 +705,26 @@ __global__ void __launch_bounds__(C::T, C::CTAS) k_bidir_log(BiArgs A) {
         const unsigned long long deep = out + ld_vol(&A.ctl->ndeep), left = count - nx;
         rest |= deep > 256 && 2 * deep > nx && (left > 4096 || left * out > 256ull * nx);
       }
+      if (C::WIDE && out) {
+        const unsigned long long lng = ld_vol(&A.ctl->nlong);
+        rest |= lng > 64 && 2 * lng > nx;
+      }
       S.item[par ^ 1] = nx;
       S.skip[par ^ 1] = rest;
     }
     __syncthreads();
     if (skip || !log_search<C>(A, S, jr, QC)) {
       if (tid == 0) {
-        A.out[atomicAdd(A.out_count, 1ull)] = jr;
-        if (C::WIDE && !skip) atomicAdd(&A.ctl->noutgrown, 1ull);
+        uint64_t e = jr;
+        if constexpr (C::WIDE)
+          if (!skip) {
+            atomicAdd(&A.ctl->noutgrown, 1ull);
+            if (S.ovf || max(S.lvl[0], S.lvl[1]) + 1 >= C::LV) {
+              atomicAdd(&A.ctl->nlong, 1ull);
+              e |= kLongId;
+            }
+          }
+        A.out[atomicAdd(A.out_count, 1ull)] = e;
       }
     } else if (tid == 0) {
       arcs += S.arcs;

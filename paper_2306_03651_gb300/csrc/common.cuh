@@ -349,7 +349,7 @@ struct cen_graph {
   // them they handed on, and whether that was most (the wide CTAs come first then).
   mutable std::atomic<uint64_t> bidir_seen{0}, bidir_handed{0};
   mutable std::atomic<bool> bidir_wide{false};
-  // Samples of a call from which such searches start with the tables in global memory.
+  // Number of such searches of a call from which they go to the tables in global memory.
   mutable std::atomic<uint64_t> bidir_many{~0ull};
   // Set once a call handed more than 30% of its warp searches on to CTAs:
   // later jobs (without an explicit setting) search with whole CTAs only.

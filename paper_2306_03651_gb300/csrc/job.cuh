@@ -64,6 +64,7 @@ struct BiCtl {
   unsigned long long nmigrate; // searches that outgrew the small table in global memory
   unsigned long long ndeep;    // deep searches (kDeepLevels) that the wide CTAs finished
   unsigned long long noutgrown; // searches that they took up and handed on
+  unsigned long long nlong;    // searches with more levels or paths than shared memory holds at any size
   int err;
   int pad;
 };
@@ -79,6 +80,7 @@ constexpr int kTierSmall = 0, kTierWide = 1, kTierGlobal = 2;
 // 1.31 and 1.19, 8,000 3.14 and 2.50; 500 x 500 (10% left) 1,000 pairs 1.57 and 2.21, 1,500 2.42 and 1.83, 8,000 6.65
 // and 4.05; 1,400 x 1,400 (78% left) 700 pairs 3.78 and 4.01, 900 4.65 and 4.20, and 2,000 x 2,000 800 pairs 5.77 and
 // 6.39, 1,000 6.98 and 7.15.  Shallow searches (R-MAT, BA) stay in shared memory however many they are.
+// What the small CTAs hand on, where that is not most, goes to the one or the other by the same numbers.
 constexpr uint64_t kDeepLevels = 12;  // levels of both balls, or arcs between a pair less one, of a deep search
 constexpr uint64_t kManyDeep = 2048;  // many, where the wide CTAs leave nothing,
 constexpr uint64_t kManyLeft = 1024;  // some,
@@ -88,6 +90,7 @@ struct BiWS {
   DevBuf tabw, epw;        // warp searches: node tables and epochs (none when WQ = 0)
   DevBuf big, far;         // ids that a launch hands on to the next (used in turn)
   int tier = 0;            // where searches by CTAs start (kTier*)
+  bool straight = false;   // what the small CTAs leave goes to the tables in global memory at once
   int nslots = 0;          // CTAs that the budget allows tables in global memory for
   int tables = 0;          // CTAs that have them (bidir_tables)
   int64_t QC = 0;
@@ -197,7 +200,8 @@ namespace cen {
 constexpr int64_t kShortMembers = 16;
 void sample_append(cen_job *job, uint64_t m_new);
 void bidir_launch(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages);
-void bidir_launch_rest(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages, uint64_t left);
+void bidir_launch_rest(cen_job *job, uint64_t j0, uint64_t count, int64_t arena_cap, int *stages, uint64_t left,
+                       bool wide);
 // Entries of each list of a warp search for a CTA queue of QC entries (0: warp searches off).
 int64_t bidir_warp_queue(int64_t QC);
 size_t bidir_warp_bytes_per_slot();

@@ -1295,9 +1295,10 @@ void bidir_setup(cen_job *job, uint64_t m_new) {
   // searches start in shared memory unless a table size was set, the ids are too long for it, or the call has
   // many of those that would not stay there
   const bool wide = job->g->bidir_wide.load();
+  const uint64_t many = job->g->bidir_many.load();
   const int tier = job->bidir_table >= 0 || !bidir_shared_ok(n)     ? kTierGlobal
                    : !wide                                          ? kTierSmall
-                   : m_new < job->g->bidir_many.load()              ? kTierWide
+                   : m_new < many                                   ? kTierWide
                                                                     : kTierGlobal;
   // By default, warp searches and small tables only where no record says that searches outgrow the
   // small CTAs (they outgrow a warp and a small table then too); warps only where frontiers grow slowly
@@ -1344,6 +1345,8 @@ void bidir_setup(cen_job *job, uint64_t m_new) {
   }
   for (DevBuf *b : {&wk.tab1, &wk.tab2, &wk.lists, &wk.sig, &wk.epochs, &wk.tabw, &wk.epw}) b->st = st;
   wk.tier = tier;
+  const double share = (double)job->g->bidir_handed.load() / (double)std::max<uint64_t>(1, job->g->bidir_seen.load());
+  wk.straight = tier == kTierSmall && share * (double)m_new >= (double)many;
   wk.ctl.ensure(sizeof(BiCtl), st);
   wk.big.ensure(8 * (size_t)m_new, st);
   wk.far.ensure(8 * (size_t)m_new, st);
@@ -1370,23 +1373,25 @@ static BiCtl bidir_search(cen_job *job, uint64_t m0, uint64_t m_new, int64_t cap
   BiCtl h = bidir_finish(job);
   const uint64_t left = h.nout[*stages - 1];
   if (!left) return h;
-  bidir_launch_rest(job, m0, m_new, cap, stages, left);
+  bidir_launch_rest(job, m0, m_new, cap, stages, left, 2 * h.nlong <= left);
   return bidir_finish(job);
 }
 
 // What a call's shared-memory searches show of the graph: whether most outgrow the small CTAs (over all calls, so
 // that short ones settle too), and then from how many samples on a call starts in global memory.
-static void bidir_record(const cen_graph *g, int tier, uint64_t m_new, const BiCtl &h) {
+static void bidir_record(const cen_graph *g, int tier, bool straight, uint64_t m_new, const BiCtl &h) {
   if (tier == kTierSmall) {
     const uint64_t handed = g->bidir_handed += h.nout[0], seen = g->bidir_seen += m_new;
     if (seen >= 512 && 2 * handed > seen) g->bidir_wide.store(true);
   }
-  if (!g->bidir_wide.load()) return;
+  if (straight) return;
   const uint64_t in = tier == kTierSmall ? h.nout[0] : m_new, left = h.nout[tier == kTierSmall ? 1 : 0];
   const uint64_t tried = in - left + h.noutgrown;  // of which the wide CTAs handed noutgrown on
   const bool deep = h.cursor >= kDeepLevels * m_new;
   uint64_t many = ~0ull;
-  if (tried >= 256 && 4 * h.noutgrown > 3 * tried)
+  if (tried >= 256 && 2 * h.noutgrown > tried && 2 * h.nlong > left)
+    many = 0;
+  else if (tried >= 256 && 4 * h.noutgrown > 3 * tried)
     many = kManyMost;
   else if (left && (deep || (tried >= 256 && 2 * h.noutgrown > tried)))
     many = kManyLeft;
@@ -1426,7 +1431,7 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   const unsigned long long nbig = bw.WQ ? h.nout[0] : 0;
   // learnt from calls whose CTA searches see every sample and have queues of full length
   if (bw.tier != kTierGlobal && !bw.WQ && job->bidir_queue >= kBidirQueue)
-    bidir_record(job->g, bw.tier, m_new, h);
+    bidir_record(job->g, bw.tier, bw.straight, m_new, h);
   if (job->bidir_warps < 0 && bw.WQ && m_new >= 1024 && 10 * nbig > 3 * m_new) job->g->bidir_warps_off.store(true);
   std::vector<uint64_t> search(h.nsearch), walk(h.nwalk);
   if (h.nsearch)
@@ -1480,7 +1485,8 @@ int64_t append_bidir(cen_job *job, uint64_t m0, uint64_t m_new) {
   job->bidir_deferred_search += h.nsearch;
   job->bidir_deferred_walk += walk.size();
   job->bidir_migrated += h.nmigrate;
-  if (bw.tier != kTierGlobal) job->bidir_migrated += h.nout[(bw.WQ ? 1 : 0) + (bw.tier == kTierSmall ? 1 : 0)];
+  if (bw.tier != kTierGlobal)
+    job->bidir_migrated += h.nout[(bw.WQ ? 1 : 0) + (bw.tier == kTierSmall && !bw.straight ? 1 : 0)];
   job->bidir_escalated += nbig;
   return total;
 }

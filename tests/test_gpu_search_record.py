@@ -1,8 +1,10 @@
 """What calls record on a graph about the sizes of bidirectional search: which launches a later call makes.
 A call that starts with the small shared-memory CTAs makes two (small, wide) or four (and two for the
 few left), one that starts with the wide ones one or three, one with the tables in global memory one."""
+import numpy as np
 import pytest
 
+import oracle as O
 from paper_2306_03651_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
@@ -58,3 +60,40 @@ def test_searches_left_untried_do_not_count_as_left_by_the_wide_ctas():
     """The first call hands nearly all on untried; the wide CTAs would leave 10%, so a call of 950 still starts there."""
     graph = P.Graph.of(I.grid_rewired(500, 500, 0.01, 1))
     assert [launches(graph, m, 1) for m in (8000, 950)] == [3, 3]
+
+
+@pytest.mark.parametrize("nodes, kernels", [(150, 2), (220, 2), (222, 2), (244, 2), (246, 3), (700, 3)])
+def test_long_thin_searches(nodes, kernels):
+    """Pairs of a cycle are up to half its length apart, and the sides grow in turn, up to LV - 1 and LV - 2 levels:
+    110 arcs fit the small CTAs' 56 levels, 122 the wide ones' 62, and more go to the 128-thread CTAs with tables in
+    global memory, not by way of the 1,024-thread ones."""
+    g = I.from_edges(nodes, np.arange(nodes), (np.arange(nodes) + 1) % nodes, False)
+    job, ojob = P.Job(P.Graph.of(g), 1, 1), O.Job(O.Graph.of(g), 1, 1)
+    job.sample(2000)
+    ojob.sample(2000)
+    assert job.stats()["bidir"]["launches"] == kernels
+    h, ref = job.samples(), ojob.hypergraph()
+    assert h["d"].max() >= nodes // 2 - 1
+    for key in ("hoff", "s", "t", "d"):
+        assert np.array_equal(h[key], ref[key]), key
+    assert np.array_equal(h["hmem"], ref["hmem"][:ref["hoff"][-1]])
+
+
+def test_deep_searches_that_small_ctas_leave_skip_the_wide_ones_where_they_are_many():
+    """Some 43% of this grid's searches outgrow the small CTAs, 3,400 of 8,000: from the second call on those go
+    straight to the tables in global memory; 1,290 of 3,000 do not."""
+    graph = P.Graph.of(I.grid_rewired(120, 120, 0.01, 1))
+    job = P.Job(graph, 2, 1)
+    job.tune(bidir_table=0, bidir_warps=0)
+    job.sample(8000)
+    for m in (8000, 8000, 3000):
+        other = P.Job(graph, 2, 1)
+        other.sample(m)
+        h, ref = other.samples(), job.samples()
+        members = int(h["hoff"][-1])
+        assert all(np.array_equal(h[key], ref[key][:len(h[key])]) for key in ("hoff", "s", "t", "d"))
+        assert np.array_equal(h["hmem"], ref["hmem"][:members])
+    assert other.sampler_info()["migrated"] == 0
+    last = P.Job(graph, 2, 1)
+    last.sample(8000)
+    assert last.stats()["bidir"]["launches"] == 2 and last.sampler_info()["migrated"] > 3000
